@@ -50,15 +50,22 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 }
 
 // Wait for the phase of `bar` with the given parity; false if it did not
-// complete within timeout_ns or another warp of the CTA already gave up.
+// complete within timeout_ns or another warp of the CTA already gave up.  The
+// clock and the flag are looked at between bursts of polls only: reading the
+// global timer takes far longer than a poll and would delay the wake-up.
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity,
                                                   uint64_t timeout_ns, volatile int* abort_flag) {
+  constexpr int kBurst = 32;
   if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = global_ns();
+  uint64_t t0 = 0;
   for (;;) {
-    if (mbar_try_wait(bar, parity)) return true;
+#pragma unroll 1
+    for (int i = 0; i < kBurst; ++i)
+      if (mbar_try_wait(bar, parity)) return true;
     if (abort_flag && *abort_flag) return false;
-    if (global_ns() - t0 > timeout_ns) return false;
+    const uint64_t t = global_ns();
+    if (t0 == 0) t0 = t;
+    else if (t - t0 > timeout_ns) return false;
   }
 }
 

@@ -1,6 +1,7 @@
-// gather.cuh -- the persistent gather kernel of Eq. (BP) and its launch
-// templates (internal).  Two translation units instantiate it: kernels.cu for
-// delays read from the stored fast-marching table, gather_const.cu for the
+// gather.cuh -- the persistent staged gather kernel of Eq. (BP) for units of 1
+// or 2 frames (plans, forced staging; gather_rows.cuh takes 4 frames and more)
+// and its launch templates (internal).  kernels.cu instantiates it for delays
+// read from the stored fast-marching table, gather_const.cu for the
 // conventional constant-speed delays computed in the kernel (Sec. II-C).
 //
 //   out[f][r] = sum_s w_s * b_{f,s}(T_s(r)/dt) with linear interpolation.
@@ -77,26 +78,10 @@ __device__ __forceinline__ void solid_angle_weights(float (&ww)[4], const float4
   for (int x = 0; x < 4; ++x) ww[x] = solid_angle_weight(pq[x], E, N);
 }
 
-// Rows of 8 frames (32 bytes, four to a 128-byte line of shared-memory banks)
-// are stored with their two 16-byte halves swapped when bit 2 of the row index
-// is set.  The 8 lanes of a 16-byte load phase read rows of 8 pixels; without
-// the swap two of them conflict whenever their rows agree mod 4, with it only
-// when they agree mod 8.  Windows start at rows that are multiples of 8 in
-// global and shared memory, so a row's swap is the same in both.
-__device__ __forceinline__ void load_row8(const uint32_t* sw, unsigned r, uint32_t (&w)[8]) {
-  const unsigned x = (r >> 2) & 1u;
-  const uint4 lo = *reinterpret_cast<const uint4*>(sw + r * 8u + 4u * x);
-  const uint4 hi = *reinterpret_cast<const uint4*>(sw + r * 8u + 4u * (x ^ 1u));
-  w[0] = lo.x; w[1] = lo.y; w[2] = lo.z; w[3] = lo.w;
-  w[4] = hi.x; w[5] = hi.y; w[6] = hi.z; w[7] = hi.w;
-}
-
-// Frames fb of row r of a window in shared memory (FB words per row; 8-frame
-// rows as load_row8 describes).
+// Frames fb of row r of a window in shared memory (FB words per row).
 template <int FB>
 __device__ __forceinline__ void load_row(const uint32_t* sw, unsigned r, uint32_t (&w)[FB]) {
-  if constexpr (FB == 8) load_row8(sw, r, w);
-  else load_words<FB>(sw + size_t(r) * FB, w);
+  load_words<FB>(sw + size_t(r) * FB, w);
 }
 
 // Interpolate one sensor's integrand at the lane's 4 window offsets uu (rows
@@ -183,17 +168,13 @@ __device__ __forceinline__ void gather_sensor(float (&acc)[FB][4], const float* 
 // Anchor of the sensor (two float4): (e.x, e.y, e.z, u0), (u0 - base, cap,
 // u0^2, flag), cap = (N_t - 1) - base; offsets above cap are after the
 // record.  Per pixel (registers): pq = (2 D.x, 2 D.y, 2 D.z, |D|^2).
-template <int FB, int FMT, int WGT>
-__device__ __forceinline__ void gather_sensor_const(float (&acc)[FB][4], const float4 (&pq)[4],
-                                                    const float4* sa, const uint32_t* sm,
-                                                    const int* soff, const uint32_t* sw, int sl,
-                                                    int Wst, const float4* swa) {
-  const float4 A = sa[2 * sl], B = sa[2 * sl + 1];
-  float uu[4];
+template <int N>
+__device__ __forceinline__ void constant_offsets(float (&uu)[N], const float4 (&pq)[N], float4 A,
+                                                 float4 B) {
   if (B.w == 0.0f) {  // the same sensor for the whole warp: a uniform branch
     const float m2u0 = -2.0f * A.w;
 #pragma unroll
-    for (int x = 0; x < 4; ++x) {
+    for (int x = 0; x < N; ++x) {
       const float num = fmaf(pq[x].x, A.x, fmaf(pq[x].y, A.y, fmaf(pq[x].z, A.z, pq[x].w)));
       const float s = num + B.z;
       const float y = rsqrtf(s);
@@ -204,7 +185,7 @@ __device__ __forceinline__ void gather_sensor_const(float (&acc)[FB][4], const f
     }
   } else {
 #pragma unroll
-    for (int x = 0; x < 4; ++x) {
+    for (int x = 0; x < N; ++x) {
       const float d0 = fmaf(0.5f, pq[x].x, A.x), d1 = fmaf(0.5f, pq[x].y, A.y),
                   d2 = fmaf(0.5f, pq[x].z, A.z);
       const float s = fmaxf(fmaf(d0, d0, fmaf(d1, d1, d2 * d2)), 1.0e-30f);
@@ -212,6 +193,15 @@ __device__ __forceinline__ void gather_sensor_const(float (&acc)[FB][4], const f
       uu[x] = v > B.y ? kFarOffset : fmaxf(v, 0.0f);
     }
   }
+}
+
+template <int FB, int FMT, int WGT>
+__device__ __forceinline__ void gather_sensor_const(float (&acc)[FB][4], const float4 (&pq)[4],
+                                                    const float4* sa, const uint32_t* sm,
+                                                    const int* soff, const uint32_t* sw, int sl,
+                                                    int Wst, const float4* swa) {
+  float uu[4];
+  constant_offsets<4>(uu, pq, sa[2 * sl], sa[2 * sl + 1]);
   float ww[4] = {1.0f, 1.0f, 1.0f, 1.0f};
   if constexpr (WGT != 0) solid_angle_weights(ww, pq, swa[2 * sl], swa[2 * sl + 1]);
   lerp_accumulate<FB, FMT, WGT>(acc, uu, ww, sm + sl * FB, soff[sl], sw, Wst);
@@ -709,8 +699,6 @@ static cudaError_t gather_fb(int FB, const StreamParams& p, size_t smem, int gri
   switch (FB) {
     case 1: return gather_t<P, 1, FMT, SW, MODE>(p, smem, grid, st, resident, n_sm);
     case 2: return gather_t<P, 2, FMT, SW, MODE>(p, smem, grid, st, resident, n_sm);
-    case 4: return gather_t<P, 4, FMT, SW, MODE>(p, smem, grid, st, resident, n_sm);
-    case 8: return gather_t<P, 8, FMT, SW, MODE>(p, smem, grid, st, resident, n_sm);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -739,8 +727,6 @@ static const void* gather_func_fb(int FB) {
   switch (FB) {
     case 1: return reinterpret_cast<const void*>(gather_kernel<P, 1, FMT, SW, MODE>);
     case 2: return reinterpret_cast<const void*>(gather_kernel<P, 2, FMT, SW, MODE>);
-    case 4: return reinterpret_cast<const void*>(gather_kernel<P, 4, FMT, SW, MODE>);
-    case 8: return reinterpret_cast<const void*>(gather_kernel<P, 8, FMT, SW, MODE>);
   }
   return nullptr;
 }

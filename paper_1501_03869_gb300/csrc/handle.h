@@ -50,8 +50,8 @@ struct pat_bp_s {
   int pre_fb = 1;                     // their frames per group
   int wst_cache[33] = {0};            // stage window bound per sensors-per-stage
   // launch shapes chosen by the autotuner: [frames-per-group index][format]
-  int tuned_S[4][3] = {};
-  int tuned_budget_kb[4][3] = {};
+  int tuned_S[6][3] = {};
+  int tuned_budget_kb[6][3] = {};
   float* d_u = nullptr;               // table offsets (delays == 0)
   float* d_anchor = nullptr;          // per (tile, sensor) anchors (delays == 1)
   float4* d_pix = nullptr;            // per-pixel terms (delays == 1 or wgt)
@@ -102,7 +102,7 @@ namespace patbp {
 // frame after the other.
 constexpr int kStagedMinFrames = 4;
 int frames_per_group(int n_frames);
-// frames per unit a handle's reconstruction of n_frames uses (1 below kStagedMinFrames)
+// frames per unit that suit a handle's reconstruction of n_frames (1 below kStagedMinFrames)
 int frames_per_unit(pat_bp_t h, int n_frames);
 int fb_index(int FB);
 int fmt_for(pat_dtype dt);
@@ -113,8 +113,14 @@ int stage_window(pat_bp_t h, int S);
 // stages and window-row budget of a shape under a smem budget (false: nothing fits)
 bool fit_stages(GatherConfig& c, int wmin, int wfull, size_t budget, int* wst);
 // launch shape: frames per unit, sensors per stage, stages under a smem budget
-GatherConfig config_for(pat_bp_t h, int FB, int S, size_t budget, int* wst);
-GatherConfig pick_config(pat_bp_t h, int n_frames, int fmt, int* wst);
+GatherConfig config_for(pat_bp_t h, int n_frames, int FB, int S, size_t budget, int* wst);
+// (max_fb caps the frames per unit)
+GatherConfig pick_config(pat_bp_t h, int n_frames, int fmt, int* wst, int max_fb = 32);
+void default_shape(int FB, size_t limit, int* S, size_t* budget);
+// whole-tile or one-segment units for a launch of `tiles` (frame group, tile) pairs
+void set_units(GatherConfig& c, int64_t tiles, int n_seg);
+// units of one instance
+int64_t unit_count(const GatherConfig& c, const InstDesc& d);
 // one instance's preprocessing and gather descriptors for n_frames frames
 PreParams make_pre(pat_bp_t h, const void* sig, pat_dtype dtype, const float* scales, int n_frames,
                    int FB);

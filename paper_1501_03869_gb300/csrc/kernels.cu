@@ -6,15 +6,18 @@
 //                      pairs with a per-row scale.  Since t_k / dt = k the
 //                      interior value is 2 p_k - k (p_{k+1} - p_{k-1}).
 //   gather_kernel      out[f][r] = sum_s w_s * b_{f,s}(T_s(r)/dt) with linear
-//                      interpolation (Sec. II-C), defined in gather.cuh; this
-//                      unit instantiates it for delays from the stored
-//                      fast-marching table and holds the launchers.
+//                      interpolation (Sec. II-C) for units of 1 or 2 frames,
+//                      defined in gather.cuh; this unit instantiates it for
+//                      delays from the stored fast-marching table and holds
+//                      the launchers of every gather (gather_rows.cuh: units
+//                      of 4 to 32 frames).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <cstdio>
 
-#include "gather.cuh"
+#include "gather_rows.cuh"
 
 namespace patbp {
 // ---------------------------------------------------------- preprocessing --
@@ -216,7 +219,7 @@ __device__ __forceinline__ void preprocess_row(const PreParams& p, int s, int g)
 // has the same bits whatever the frames per group.
 template <int DT, int FMT, int FB>
 __device__ __forceinline__ void preprocess_row_frames(const PreParams& p, int s, int g) {
-  static_assert(FB >= 2 && FB <= 16 && (FB & (FB - 1)) == 0, "frames per group");
+  static_assert(FB >= 2 && FB <= 4 && (FB & (FB - 1)) == 0, "frames per group");
   constexpr int K = 8;
   constexpr int RUNS = 256 / FB;  // runs of one frame per block pass
   __shared__ float red[8][FB];
@@ -286,21 +289,234 @@ __device__ __forceinline__ void preprocess_row_frames(const PreParams& p, int s,
         if constexpr (FMT == kBF32) wv = __float_as_uint(b[j]);
         else wv = encode_pair<FMT>(b[j], b[j + 1], inv);
       }
-      // 8-frame rows: the two 16-byte halves of rows with bit 2 of the row
-      // index set are stored swapped (k0 is a multiple of 8, so that bit is
-      // j's), which the gather's shared-memory reads undo (row_half_swap)
-      const int pos = FB == 8 ? (fb ^ (((j >> 2) & 1) << 2)) : fb;
-      dst[int64_t(k0 + j) * FB + pos] = wv;
+      dst[int64_t(k0 + j) * FB + fb] = wv;
     }
   }
   if (threadIdx.x < FB) p.m[(int64_t(g) * p.n_sensors_pad + s) * FB + fb] = live ? p.weights[s] * sigma : 0.0f;
 }
 
-// One (sensor, frame group) row per CTA: the frame-fast layout for groups of
-// several frames, the sample-run layout (preprocess_row) for single frames.
+// Eq. (BP) integrand b_k of one row of n samples from p_{k-1}, p_k, p_{k+1}
+// (explicitly rounded, the expression of the two layouts above).
+__device__ __forceinline__ float integrand(int k, int n, float pm, float p0, float p1) {
+  if (k >= n) return 0.0f;
+  if (k == 0) return 2.0f * p0;
+  if (k == n - 1) return fmaf(-2.0f * float(k), __fsub_rn(p0, pm), 2.0f * p0);
+  return fmaf(-float(k), __fsub_rn(p1, pm), 2.0f * p0);
+}
+
+// Two 16-bit samples of a word as FP32 (low half first).
+template <int DT>
+__device__ __forceinline__ float2 unpack_samples(uint32_t w) {
+  if constexpr (DT == 1) return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+  else return __half22float2(*reinterpret_cast<const __half2*>(&w));
+}
+
+// Codes of samples k0 .. k0 + 7 of a 16-bit row, zero outside [0, n).
+__device__ __forceinline__ uint4 load_codes8(const uint16_t* row, int k0, int n) {
+  const uint16_t* ptr = row + k0;
+  if (k0 >= 0 && k0 + 8 <= n && (reinterpret_cast<uintptr_t>(ptr) & 15) == 0)
+    return __ldg(reinterpret_cast<const uint4*>(ptr));
+  uint32_t w[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int k = k0 + 2 * j;
+    const uint32_t lo = k >= 0 && k < n ? __ldg(row + k) : 0u, hi = k + 1 >= 0 && k + 1 < n ? __ldg(row + k + 1) : 0u;
+    w[j] = lo | hi << 16;
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// Rows of 8, 16 or 32 frames per group.  A row of FB frames is contiguous, so
+// frames must be fastest across the lanes for the stores while the signals are
+// contiguous in time: chunks of KC samples of all frames go through shared
+// memory (odd pitches keep both sides nearly free of bank conflicts), the next
+// chunk's loads in flight while one is computed.  Bound by HBM for FP32 (64
+// paper-shaped frames: 538 MB); by instruction issue for 16-bit signals, whose
+// integrands need the row's largest |b| first: a pass over the signals with a
+// warp per frame (the second pass finds them in L2).  part of parts: the share
+// of the row's chunks that this CTA writes (short launches split rows to fill
+// the chip; each share repeats the first pass).
 template <int DT, int FMT, int FB>
-__device__ __forceinline__ void preprocess_group(const PreParams& p, int s, int g) {
+__device__ __forceinline__ void preprocess_row_tiles(const PreParams& p, int s, int g, int part, int parts) {
+  static_assert(FB == 8 || FB == 16 || FB == 32, "frames per group");
+  constexpr int KC = 4096 / FB, COLS = KC + 4;            // samples c0 - 2 .. c0 + KC + 1
+  constexpr int W = DT == 0 ? 1 : 2;                      // samples of one word
+  constexpr int WORDS = COLS / W, PITCH = WORDS + 1;      // odd
+  constexpr int RUNS = 256 / FB, RUN = KC / RUNS;         // 16 samples per thread and chunk
+  constexpr int NF = FB / 8;                              // frames of a warp
+  constexpr int NL = (WORDS + 31) / 32;                   // loads per frame and lane
+  __shared__ uint32_t tile[FB][PITCH];
+  __shared__ float sig_s[FB];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int f0 = g * FB, live = min(FB, p.n_frames - f0), n = p.n_t;
+  const int fb = threadIdx.x & (FB - 1), run = threadIdx.x / FB;
+  int64_t row0[NF];
+#pragma unroll
+  for (int i = 0; i < NF; ++i) row0[i] = (int64_t(f0 + min(warp + 8 * i, live - 1)) * p.n_sensors + s) * n;
+  const float sc = p.scales && fb < live ? p.scales[int64_t(f0 + fb) * p.n_sensors + s] : 1.0f;
+  float sigma = 1.0f, inv = 1.0f;
+  if constexpr (FMT != kBF32) {
+    // largest |b| per frame: 8 samples per lane and step, UN steps in flight
+    constexpr int UN = 4 / NF;
+    float mx[NF], scf[NF];
+#pragma unroll
+    for (int i = 0; i < NF; ++i) {
+      mx[i] = 0.0f;
+      scf[i] = p.scales ? p.scales[row0[i] / n] : 1.0f;
+    }
+    for (int kw = 0; kw < n; kw += 256 * UN) {
+      uint4 raw[UN][NF];
+      uint32_t edge[UN][NF];  // the sample before lane 0's, after lane 31's
+#pragma unroll
+      for (int u = 0; u < UN; ++u)
+#pragma unroll
+        for (int i = 0; i < NF; ++i) {
+          const uint16_t* row = static_cast<const uint16_t*>(p.sig) + row0[i];
+          const int k0 = kw + u * 256 + lane * 8, ke = lane == 0 ? k0 - 1 : k0 + 8;
+          raw[u][i] = load_codes8(row, k0, n);
+          edge[u][i] = (lane == 0 || lane == 31) && ke >= 0 && ke < n ? __ldg(row + ke) : 0u;
+        }
+#pragma unroll
+      for (int u = 0; u < UN; ++u)
+#pragma unroll
+        for (int i = 0; i < NF; ++i) {
+          const int k0 = kw + u * 256 + lane * 8;
+          const uint32_t w[4] = {raw[u][i].x, raw[u][i].y, raw[u][i].z, raw[u][i].w};
+          float v[10];  // p_{k0-1} .. p_{k0+8}
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float2 x = unpack_samples<DT>(w[j]);
+            v[1 + 2 * j] = __fmul_rn(x.x, scf[i]);
+            v[2 + 2 * j] = __fmul_rn(x.y, scf[i]);
+          }
+          const float e = __fmul_rn(unpack_samples<DT>(edge[u][i]).x, scf[i]);
+          const float prev = __shfl_up_sync(0xffffffffu, v[8], 1), nxt = __shfl_down_sync(0xffffffffu, v[1], 1);
+          v[0] = lane == 0 ? e : prev;
+          v[9] = lane == 31 ? e : nxt;
+          if (k0 > 0 && k0 + 8 < n) {
+            const float kf = -float(k0);
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              mx[i] = fmaxf(mx[i], fabsf(fmaf(kf - float(j), __fsub_rn(v[j + 2], v[j]), 2.0f * v[j + 1])));
+          } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) mx[i] = fmaxf(mx[i], fabsf(integrand(k0 + j, n, v[j], v[j + 1], v[j + 2])));
+          }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < NF; ++i) {
+      for (int o = 16; o > 0; o >>= 1) mx[i] = fmaxf(mx[i], __shfl_xor_sync(0xffffffffu, mx[i], o));
+      if (lane == 0) sig_s[warp + 8 * i] = mx[i] > 0.0f ? mx[i] : 1.0f;
+    }
+    __syncthreads();
+    sigma = sig_s[fb];
+    inv = 1.0f / sigma;
+  }
+  // 16-bit signals go two samples per load when every row starts on 4 bytes
+  const bool pairs = W == 2 && (n & 1) == 0 && (reinterpret_cast<uintptr_t>(p.sig) & 3) == 0;
+  uint32_t raw[NF][NL];
+  auto fetch = [&](int c0) {
+    const bool whole = c0 > 0 && c0 + KC + 2 <= n && (W == 1 || pairs);
+#pragma unroll
+    for (int i = 0; i < NF; ++i) {
+      const bool on = warp + 8 * i < live;  // absent frames are stored as zeros
+#pragma unroll
+      for (int l = 0; l < NL; ++l) {
+        const int q = l * 32 + lane, k = c0 - 2 + W * q;
+        uint32_t w = 0u;
+        if constexpr (DT == 0) {
+          const float* src = static_cast<const float*>(p.sig) + row0[i] + k;
+          if (on && q < WORDS && (whole || (k >= 0 && k < n))) w = __float_as_uint(__ldg(src));
+        } else {
+          const uint16_t* src = static_cast<const uint16_t*>(p.sig) + row0[i] + k;
+          if (whole) {
+            if (on && q < WORDS) w = __ldg(reinterpret_cast<const uint32_t*>(src));
+          } else if (on && q < WORDS && k >= 0 && k < n) {
+            if (pairs) w = __ldg(reinterpret_cast<const uint32_t*>(src));
+            else w = uint32_t(__ldg(src)) | (k + 1 < n ? uint32_t(__ldg(src + 1)) << 16 : 0u);
+          }
+        }
+        raw[i][l] = w;
+      }
+    }
+  };
+  uint32_t* dst = static_cast<uint32_t*>(p.b) + (int64_t(g) * p.n_sensors + s) * p.n_t_pad * FB + fb;
+  const int chunks = (p.n_t_pad + KC - 1) / KC;
+  const int cb = int(int64_t(chunks) * part / parts) * KC, ce = int(int64_t(chunks) * (part + 1) / parts) * KC;
+  if (cb < ce) fetch(cb);
+  for (int c0 = cb; c0 < ce; c0 += KC) {
+    if (c0 != cb) __syncthreads();  // the chunk before has been read
+#pragma unroll
+    for (int i = 0; i < NF; ++i)
+#pragma unroll
+      for (int l = 0; l < NL; ++l)
+        if (l * 32 + lane < WORDS) tile[warp + 8 * i][l * 32 + lane] = raw[i][l];
+    __syncthreads();
+    if (c0 + KC < ce) fetch(c0 + KC);
+    const uint32_t* row = tile[fb] + run * RUN / W;  // the word of p_{k0-2}
+    const int k0 = c0 + run * RUN;
+    if (k0 >= p.n_t_pad) continue;
+    uint32_t* out = dst + int64_t(k0) * FB;
+    // p_{k0-1}, p_{k0}, p_{k0+1}, then p_{k+2} for k = k0, k0 + 1, ..
+    float pm, pc, pn, later = 0.0f;
+    if constexpr (W == 1) {
+      pm = __fmul_rn(__uint_as_float(row[1]), sc);
+      pc = __fmul_rn(__uint_as_float(row[2]), sc);
+      pn = __fmul_rn(__uint_as_float(row[3]), sc);
+    } else {
+      const float2 x = unpack_samples<DT>(row[0]), y = unpack_samples<DT>(row[1]);
+      pm = __fmul_rn(x.y, sc);
+      pc = __fmul_rn(y.x, sc);
+      pn = __fmul_rn(y.y, sc);
+    }
+    auto ahead = [&](int j) {  // p_{k0 + j + 2}
+      if constexpr (W == 1) return __fmul_rn(__uint_as_float(row[j + 4]), sc);
+      if (j & 1) return later;
+      const float2 x = unpack_samples<DT>(row[j / 2 + 2]);
+      later = __fmul_rn(x.y, sc);
+      return __fmul_rn(x.x, sc);
+    };
+    if (k0 > 0 && k0 + RUN + 1 < n) {  // inside the record: one expression
+      float kf = -float(k0);
+      float b = fmaf(kf, __fsub_rn(pn, pm), 2.0f * pc);
+#pragma unroll
+      for (int j = 0; j < RUN; ++j) {
+        const float pn2 = ahead(j);
+        const float b1 = fmaf(kf - float(j + 1), __fsub_rn(pn2, pc), 2.0f * pn);
+        if constexpr (FMT == kBF32) out[j * FB] = __float_as_uint(b);
+        else out[j * FB] = encode_pair<FMT>(b, b1, inv);
+        b = b1;
+        pc = pn;
+        pn = pn2;
+      }
+    } else {
+      float b = integrand(k0, n, pm, pc, pn);
+#pragma unroll
+      for (int j = 0; j < RUN; ++j) {
+        const float pn2 = ahead(j);
+        const float b1 = integrand(k0 + j + 1, n, pc, pn, pn2);
+        uint32_t wv;
+        if constexpr (FMT == kBF32) wv = __float_as_uint(b);
+        else wv = encode_pair<FMT>(b, b1, inv);
+        if (k0 + j < p.n_t_pad) out[j * FB] = wv;
+        b = b1;
+        pc = pn;
+        pn = pn2;
+      }
+    }
+  }
+  if (part == 0 && threadIdx.x < FB)
+    p.m[(int64_t(g) * p.n_sensors_pad + s) * FB + fb] = fb < live ? p.weights[s] * sigma : 0.0f;
+}
+
+// One (sensor, frame group) row per CTA: the sample-run layout for single
+// frames, the frame-fast one for 2 and 4, tiles for 8, 16 and 32.
+template <int DT, int FMT, int FB>
+__device__ __forceinline__ void preprocess_group(const PreParams& p, int s, int g, int part = 0,
+                                                 int parts = 1) {
   if constexpr (FB == 1) preprocess_row<DT, FMT, FB>(p, s, g);
+  else if constexpr (FB >= 8) preprocess_row_tiles<DT, FMT, FB>(p, s, g, part, parts);
   else preprocess_row_frames<DT, FMT, FB>(p, s, g);
 }
 
@@ -308,7 +524,7 @@ template <int DT, int FMT, int FB>
 __global__ void __launch_bounds__(256) preprocess_kernel(const PreParams p) {
   // let the gather that depends on this kernel start its prologue now
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  preprocess_group<DT, FMT, FB>(p, blockIdx.x, blockIdx.y);
+  preprocess_group<DT, FMT, FB>(p, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.z);
 }
 
 // Several instances in one launch: CTA x belongs to the instance whose range
@@ -353,9 +569,9 @@ __global__ void wait_probe_kernel(int* status, uint64_t timeout_ns) {
 }
 
 // --------------------------------------------------------------- launchers --
-int gather_threads(const GatherConfig& c) { return 32 * ((c.P / 128) * c.SW + 3); }
-
 size_t gather_smem_bytes(const GatherConfig& c, int Wst) {
+  if (c.FB >= 4)  // the ring, two zero rows and the running sums
+    return size_t(kRowsHeader) + c.ring + 2 * c.FB * 4 + (c.total ? size_t(c.P) * c.FB * 4 : 0);
   const StageLayout L(c.S, c.P, c.FB, Wst, c.delays | (c.wgt << 1));
   return size_t(kHeaderBytes) + kMetaBytes + L.bytes * c.stages + 2 * size_t(c.SW) * c.FB * c.P * 4;
 }
@@ -363,11 +579,18 @@ size_t gather_smem_bytes(const GatherConfig& c, int Wst) {
 template <int DT, int FMT>
 static cudaError_t launch_pre_fb(const PreParams& p, cudaStream_t st) {
   dim3 grid(p.n_sensors, (p.n_frames + p.FB - 1) / p.FB);
+  // tiles: rows are split in time while that fills the chip (4 CTAs per SM)
+  if (p.FB >= 8) {
+    const int64_t chunks = (int64_t(p.n_t_pad) * p.FB + 4095) / 4096, rows = int64_t(grid.x) * grid.y;
+    grid.z = unsigned(std::max<int64_t>(1, std::min<int64_t>(chunks, 4 * 152 / rows)));
+  }
   switch (p.FB) {
     case 1: preprocess_kernel<DT, FMT, 1><<<grid, 256, 0, st>>>(p); break;
     case 2: preprocess_kernel<DT, FMT, 2><<<grid, 256, 0, st>>>(p); break;
     case 4: preprocess_kernel<DT, FMT, 4><<<grid, 256, 0, st>>>(p); break;
     case 8: preprocess_kernel<DT, FMT, 8><<<grid, 256, 0, st>>>(p); break;
+    case 16: preprocess_kernel<DT, FMT, 16><<<grid, 256, 0, st>>>(p); break;
+    case 32: preprocess_kernel<DT, FMT, 32><<<grid, 256, 0, st>>>(p); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -383,6 +606,8 @@ static cudaError_t launch_pre_multi_fb(const PreMultiParams& p, cudaStream_t st)
     case 2: preprocess_multi_kernel<DT, FMT, 2><<<grid, 256, 0, st>>>(p); break;
     case 4: preprocess_multi_kernel<DT, FMT, 4><<<grid, 256, 0, st>>>(p); break;
     case 8: preprocess_multi_kernel<DT, FMT, 8><<<grid, 256, 0, st>>>(p); break;
+    case 16: preprocess_multi_kernel<DT, FMT, 16><<<grid, 256, 0, st>>>(p); break;
+    case 32: preprocess_multi_kernel<DT, FMT, 32><<<grid, 256, 0, st>>>(p); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -409,8 +634,68 @@ cudaError_t launch_preprocess(const PreParams& p, cudaStream_t st) {
   return cudaErrorInvalidValue;
 }
 
+static cudaError_t rows_dispatch(const GatherConfig& c, int fmt, const StreamParams* p, int grid,
+                                 cudaStream_t st, int* resident, const void** func) {
+  const size_t smem = p ? gather_smem_bytes(c, p->Wst) : 0;
+  if (c.wgt)
+    return c.delays ? rows_dispatch_3(c, fmt, p, smem, grid, st, resident, func)
+                    : rows_dispatch_2(c, fmt, p, smem, grid, st, resident, func);
+  return c.delays ? rows_dispatch_1(c, fmt, p, smem, grid, st, resident, func)
+                  : rows_dispatch_0(c, fmt, p, smem, grid, st, resident, func);
+}
+
+size_t rows_group_bytes(const GatherConfig& c, int rows) {
+  return RowsGroup(c.S, c.P, c.FB, c.delays | (c.wgt << 1)).bytes(rows, c.FB);
+}
+
+const void* rows_reduce_func(int FB) {
+  switch (FB) {
+    case 4: return reinterpret_cast<const void*>(rows_reduce_kernel<4>);
+    case 8: return reinterpret_cast<const void*>(rows_reduce_kernel<8>);
+    case 16: return reinterpret_cast<const void*>(rows_reduce_kernel<16>);
+    case 32: return reinterpret_cast<const void*>(rows_reduce_kernel<32>);
+  }
+  return nullptr;
+}
+
+bool rows_needs_reduce(const StreamParams& p) {
+  for (int i = 0; i < p.n_inst; ++i)
+    if (p.split && p.inst[i].n_seg > 1) return true;
+  return false;
+}
+
+template <int FB>
+static cudaError_t launch_rows_reduce(const StreamParams& p, int P, int n_sm, cudaStream_t st) {
+  int64_t n = 0;  // threads: one per pixel and 4 frames
+  for (int i = 0; i < p.n_inst; ++i) n += int64_t(p.inst[i].n_fg) * p.inst[i].n_tiles * P * (FB / 4);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned(std::min<int64_t>((n + 255) / 256, int64_t(n_sm) * 8)));
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, rows_reduce_kernel<FB>, p, P);
+}
+
+static cudaError_t launch_rows(const GatherConfig& c, int fmt, const StreamParams& p, int grid,
+                               cudaStream_t st) {
+  cudaError_t e = rows_dispatch(c, fmt, &p, grid, st, nullptr, nullptr);
+  if (e != cudaSuccess || !rows_needs_reduce(p)) return e;
+  switch (c.FB) {
+    case 4: return launch_rows_reduce<4>(p, c.P, c.n_sm, st);
+    case 8: return launch_rows_reduce<8>(p, c.P, c.n_sm, st);
+    case 16: return launch_rows_reduce<16>(p, c.P, c.n_sm, st);
+    case 32: return launch_rows_reduce<32>(p, c.P, c.n_sm, st);
+  }
+  return cudaErrorInvalidValue;
+}
+
 static cudaError_t gather_dispatch(const GatherConfig& c, int fmt, const StreamParams& p, int grid,
                                    cudaStream_t st, int* resident, int n_sm) {
+  if (c.FB >= 4) return rows_dispatch(c, fmt, &p, grid, st, resident, nullptr);
   if (c.wgt)
     return c.delays ? gather_dispatch_wgt_const(c, fmt, p, grid, st, resident, n_sm)
                     : gather_dispatch_wgt(c, fmt, p, grid, st, resident, n_sm);
@@ -428,11 +713,11 @@ int gather_resident_ctas(const GatherConfig& c, int fmt, int Wst, int n_sm) {
 
 cudaError_t launch_gather(const GatherConfig& c, int fmt, const StreamParams& p, int grid,
                           cudaStream_t st) {
-  if (p.stages < 1 || p.stages > kMaxStages || p.S % 4 || p.S % c.SW || p.S > kMaxS ||
+  if (p.stages < 1 || p.stages > kMaxStages || p.S < 1 || (c.FB < 4 && (p.S % 4 || p.S % c.SW)) || p.S > kMaxS ||
       p.Wst % 8 || p.n_inst < 1 || p.n_inst > kMaxInst || grid < 1)
     return cudaErrorInvalidValue;
   for (int i = 0; i < p.n_inst; ++i)
-    if (p.inst[i].G % p.S || p.inst[i].G > kMaxG || p.inst[i].Wst > p.Wst) return cudaErrorInvalidValue;
+    if ((c.FB >= 4 && p.inst[i].G > 64) || p.inst[i].G % p.S || p.inst[i].G > kMaxG || p.inst[i].Wst > p.Wst) return cudaErrorInvalidValue;
   if (p.n_units == 0) return cudaSuccess;
   if (c.direct) {
     // one frame after the other: frame f's integrand rows and multipliers are
@@ -453,10 +738,19 @@ cudaError_t launch_gather(const GatherConfig& c, int fmt, const StreamParams& p,
     }
     return cudaSuccess;
   }
+  if (c.FB >= 4) {
+    // any group of the launch must fit the ring
+    if (p.ring != c.ring || p.ring % 128 || p.S > kRowsMaxS || rows_group_bytes(c, p.Wst) > size_t(p.ring)) return cudaErrorInvalidValue;
+    return launch_rows(c, fmt, p, grid, st);
+  }
   return gather_dispatch(c, fmt, p, grid, st, nullptr, 0);
 }
 
 const void* gather_kernel_func(const GatherConfig& c, int fmt) {
+  if (c.FB >= 4) {
+    const void* f = nullptr;
+    return rows_dispatch(c, fmt, nullptr, 0, nullptr, nullptr, &f) == cudaSuccess ? f : nullptr;
+  }
   if (c.wgt) return c.delays ? gather_func_wgt_const(c, fmt) : gather_func_wgt(c, fmt);
   return c.delays ? gather_func_const(c, fmt) : gather_func_t<0>(c, fmt);
 }
@@ -468,6 +762,8 @@ static const void* pre_multi_func_fb(int FB) {
     case 2: return reinterpret_cast<const void*>(preprocess_multi_kernel<DT, FMT, 2>);
     case 4: return reinterpret_cast<const void*>(preprocess_multi_kernel<DT, FMT, 4>);
     case 8: return reinterpret_cast<const void*>(preprocess_multi_kernel<DT, FMT, 8>);
+    case 16: return reinterpret_cast<const void*>(preprocess_multi_kernel<DT, FMT, 16>);
+    case 32: return reinterpret_cast<const void*>(preprocess_multi_kernel<DT, FMT, 32>);
   }
   return nullptr;
 }

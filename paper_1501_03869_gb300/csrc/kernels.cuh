@@ -73,6 +73,9 @@ struct StreamParams {
   int S;                    // sensors per pipeline stage (multiple of 4 and of SW, <= 32)
   int stages;               // pipeline depth
   int Wst;                  // window rows one stage can need (max over instances)
+  int ring;                 // batched gather: bytes of the shared-memory ring
+  int split;                // batched gather: 1 = a unit is one segment of a tile (their sums
+                            // are added by a second kernel), 0 = all segments of a tile
   int* status;
   int* host_status;         // host-mapped word the unstaged path's last kernel copies the
                             // status into, or NULL
@@ -82,19 +85,23 @@ struct StreamParams {
 
 struct GatherConfig {
   int P = 128;      // pixels per tile
-  int FB = 1;       // frames per unit (1, 2, 4, 8)
+  int FB = 1;       // frames per unit (1, 2: gather.cuh; 4, 8, 16, 32: gather_rows.cuh)
   int SW = 4;       // sensor-phase warps
   int S = 16;       // sensors per stage
   int stages = 4;
   int delays = 0;   // 0 stored table, 1 constant speed computed in the kernel
   int wgt = 0;      // 1: solid-angle weights per (pixel, sensor)
   int direct = 0;   // 1: single frame through the unstaged kernels (gather_direct.cu)
+  int ring = 0;     // StreamParams::ring
+  int split = 0;    // StreamParams::split
+  int total = 0;    // 1: units cover several segments and keep their sum in shared memory
   int no_window = 0;  // 1: the unstaged kernel gathers from L2, never from shared-memory windows
   int n_sm = 0;     // multiprocessors of the device (sizes the unstaged grid)
 };
 
 size_t gather_smem_bytes(const GatherConfig& c, int Wst);
-int gather_threads(const GatherConfig& c);
+// Ring bytes of a batched gather's group of S sensors with `rows` window rows.
+size_t rows_group_bytes(const GatherConfig& c, int rows);
 // CTAs of one gather launch that fit on the device at once.
 int gather_resident_ctas(const GatherConfig& c, int fmt, int Wst, int n_sm);
 
@@ -106,6 +113,10 @@ cudaError_t launch_status_export(const int* status, int* host_status, cudaStream
 cudaError_t launch_preprocess_multi(const PreMultiParams& p, cudaStream_t st);
 const void* gather_kernel_func(const GatherConfig& c, int fmt);
 const void* preprocess_multi_func(int dtype, int fmt, int FB);
+// The kernel that adds the segment sums of a split launch (arguments: the
+// StreamParams, then P).
+const void* rows_reduce_func(int FB);
+bool rows_needs_reduce(const StreamParams& p);
 cudaError_t launch_gather(const GatherConfig& c, int fmt, const StreamParams& p, int grid,
                           cudaStream_t st);
 cudaError_t launch_wait_probe(int* status, uint64_t timeout_ns, cudaStream_t st);

@@ -75,7 +75,8 @@ extern "C" pat_status pat_bp_reconstruct_noalloc(pat_bp_t h, const void* signals
   PAT_CUDA(cudaSetDevice(h->device));
   const int fmt = fmt_for(dtype);
   int wst = 0;
-  const GatherConfig c = pick_config(h, n_frames, fmt, &wst);
+  // at most 8 frames per unit: the scratch limit then admits what it always did
+  const GatherConfig c = pick_config(h, n_frames, fmt, &wst, 8);
   const int FB = c.FB;
   const size_t n_fg = size_t((n_frames + FB - 1) / FB);
 
@@ -116,7 +117,9 @@ extern "C" pat_status pat_bp_reconstruct_noalloc(pat_bp_t h, const void* signals
   sp.inst[0].part = part;
   sp.inst[0].counter = counter;
   sp.n_inst = 1;
-  sp.n_units = int64_t(sp.inst[0].n_fg) * sp.inst[0].n_tiles * sp.inst[0].n_seg;
+  sp.n_units = unit_count(c, sp.inst[0]);
+  sp.split = c.split;
+  sp.ring = c.ring;
   sp.S = c.S;
   sp.stages = c.stages;
   sp.Wst = wst;

@@ -367,16 +367,44 @@ namespace patbp {
 
 int fmt_for(pat_dtype dt) { return dt == PAT_F32 ? kBF32 : (dt == PAT_BF16 ? kBBF16P : kBF16P); }
 
+// Frames per unit of a batch: the longest rows that need no more frame slots
+// (and so no larger buffers) than groups of 8.
 int frames_per_group(int n_frames) {
+  const int slots = round_up(n_frames, 8);
+  if (n_frames > 16 && round_up(n_frames, 32) <= slots) return 32;
+  if (n_frames > 8 && round_up(n_frames, 16) <= slots) return 16;
   return n_frames >= 8 ? 8 : (n_frames >= 4 ? 4 : (n_frames >= 2 ? 2 : 1));
 }
 
 int frames_per_unit(pat_bp_t h, int n_frames) {
   if (n_frames < kStagedMinFrames && !(h->flags & PAT_FLAG_STAGED_SINGLE)) return 1;
-  return frames_per_group(n_frames);
+  // Long rows make few units: shorter ones where the launch would have fewer
+  // than four units per SM (8-frame rows: one), down to 4 frames.  64 BF16
+  // frames of 6 092 pixels x 64 sensors: 41 us in rows of 32 (96 units), 34 of
+  // 16, 32 of 8, 43 of 4; 5 000 pixels x 256 sensors: 157, 121, 139, 125.
+  int FB = frames_per_group(n_frames);
+  while (FB > 4) {
+    const int64_t units = int64_t((n_frames + FB - 1) / FB) * h->n_tiles * h->n_seg;
+    if (units >= int64_t(FB == 8 ? 1 : 4) * h->n_sm) break;
+    FB /= 2;
+  }
+  return FB;
 }
 
-int fb_index(int FB) { return FB == 1 ? 0 : (FB == 2 ? 1 : (FB == 4 ? 2 : 3)); }
+int fb_index(int FB) {
+  int i = 0;
+  while ((1 << i) < FB) ++i;
+  return i;
+}
+
+// Units of the batched gather: whole tiles (all segments of G sensors) when
+// every resident CTA gets at least 8 of them, else one segment of a tile.
+void set_units(GatherConfig& c, int64_t tiles, int n_seg) {
+  if (c.FB < 4) return;
+  const int per_sm = c.FB == 32 ? 1 : (c.FB == 16 ? 2 : 4);
+  c.split = n_seg > 1 && tiles < int64_t(8) * per_sm * c.n_sm ? 1 : 0;
+  c.total = n_seg > 1 && !c.split;
+}
 
 static pat_status grow_zeroed(void** p, size_t* cap, size_t need, const char* what) {
   if (need <= *cap) return PAT_OK;
@@ -415,19 +443,24 @@ pat_status ensure_buffers_fb(pat_bp_t h, int n_frames, int FB) {
 // Largest sum of window lengths over the S-sensor stages of any tile: the
 // window rows one pipeline stage must hold.
 int stage_window(pat_bp_t h, int S) {
-  if (S >= 1 && S <= 32 && h->wst_cache[S]) return h->wst_cache[S];
-  int best = 8;
+  if (S < 1 || S > 32 || (S & (S - 1))) return 0;  // shapes use powers of two
+  if (h->wst_cache[S]) return h->wst_cache[S];
+  int best[6] = {8, 8, 8, 8, 8, 8};  // one pass for groups of 1, 2, 4, .. 32
   for (int t = 0; t < h->n_tiles; ++t) {
     const uint16_t* len = h->win_len.data() + size_t(t) * h->ns;
-    for (int s0 = 0; s0 < h->ns; s0 += S) {
-      int sum = 0;
-      for (int s = s0; s < std::min(h->ns, s0 + S); ++s) sum += len[s];
-      best = std::max(best, sum);
+    for (int s0 = 0; s0 < h->ns; s0 += 32) {
+      int sum[32];
+      for (int k = 0; k < 32; ++k) sum[k] = s0 + k < h->ns ? len[s0 + k] : 0;
+      for (int l = 0, n = 32; l < 6; ++l, n >>= 1) {
+        int m = best[l];
+        for (int k = 0; k < n; ++k) m = std::max(m, sum[k]);
+        best[l] = m;
+        for (int k = 0; k < n / 2; ++k) sum[k] = sum[2 * k] + sum[2 * k + 1];
+      }
     }
   }
-  best = round_up(best, 8);
-  if (S >= 1 && S <= 32) h->wst_cache[S] = best;
-  return best;
+  for (int l = 0; l < 6; ++l) h->wst_cache[1 << l] = round_up(best[l], 8);
+  return h->wst_cache[S];
 }
 
 // Stages and window-row budget of a launch shape under a shared-memory
@@ -437,6 +470,18 @@ int stage_window(pat_bp_t h, int S) {
 // stages down to 3) whose row budget keeps at least half of wfull wins, else
 // two stages with whatever fits above wmin.  False if even that does not fit.
 bool fit_stages(GatherConfig& c, int wmin, int wfull, size_t budget, int* wst) {
+  if (c.FB >= 4) {
+    // the whole budget is one ring; any group of S sensors must fit it (wfull
+    // rows, the longest sum over the S-sensor groups)
+    c.stages = 1;
+    c.ring = 0;
+    const size_t fixed = gather_smem_bytes(c, 0), need = rows_group_bytes(c, wfull);
+    c.ring = int(budget > fixed ? (budget - fixed) & ~size_t(127) : 0);
+    *wst = wfull;
+    if (c.ring >= int(need)) return true;
+    c.ring = int(need);
+    return false;
+  }
   for (c.stages = 6; c.stages >= 2; --c.stages) {
     const size_t fixed = gather_smem_bytes(c, 0);       // everything but the window rows
     const size_t per_row = size_t(c.stages) * c.FB * 4;  // one more row in every stage
@@ -456,7 +501,7 @@ bool fit_stages(GatherConfig& c, int wmin, int wfull, size_t budget, int* wst) {
 
 // Launch shape under a shared-memory budget: stages and row budget as
 // fit_stages decides; fewer sensors per stage if nothing fits.
-GatherConfig config_for(pat_bp_t h, int FB, int S, size_t budget, int* wst) {
+GatherConfig config_for(pat_bp_t h, int n_frames, int FB, int S, size_t budget, int* wst) {
   GatherConfig c;
   c.P = h->P;
   c.SW = h->SW;
@@ -465,43 +510,60 @@ GatherConfig config_for(pat_bp_t h, int FB, int S, size_t budget, int* wst) {
   c.n_sm = h->n_sm;
   c.FB = FB;
   c.S = S;
+  set_units(c, int64_t((n_frames + FB - 1) / FB) * h->n_tiles, h->n_seg);
   const int wmin = stage_window(h, 1);
+  if (FB >= 4) c.S = std::min(S, 16);
   for (;;) {
-    if (fit_stages(c, wmin, stage_window(h, c.S), budget, wst) || c.S <= 4) break;
-    c.S = c.S > 8 ? c.S - 8 : 4;
+    if (fit_stages(c, wmin, stage_window(h, c.S), budget, wst)) break;
+    if (FB >= 4 && c.S > 1) {
+      c.S /= 2;
+      continue;
+    }
+    if (c.S <= 4) break;
+    c.S /= 2;
   }
   return c;
 }
 
+// Sensors per group (stage) and shared-memory budget of an untuned launch.
+// Batched gather, measured on 152 SMs: rows of 16 and 32 frames take the whole
+// SM (one CTA of 8 consumer warps; half the ring is 1.2 to 1.8 times slower),
+// 8-frame rows three CTAs of 4 consumer warps (8 frames of 1.04 M voxels,
+// BF16: 2.12 ms; two CTAs 2.60, four 2.41).
+void default_shape(int FB, size_t limit, int* S, size_t* budget) {
+  static const int s[6] = {16, 8, 8, 4, 8, 4}, kb[6] = {72, 100, 72, 72, 0, 0};
+  const int i = fb_index(FB);
+  *S = s[i];
+  *budget = kb[i] ? size_t(kb[i]) * 1024 : limit;
+}
+
 // Launch shape for a frame count: the autotuned one when the handle has it,
-// else frames per unit by count, 16 (1 frame) or 8 sensors per stage and a
-// shared-memory budget of three (1 frame) or two CTAs per SM.  When the stage windows are too
-// long for that budget, the budget grows to the device limit and then fewer
+// else frames per unit by count and the default shape.  When the windows are
+// too long for its budget, the budget grows to the device limit and then fewer
 // frames share a unit.  No choice here changes the summation order.
-GatherConfig pick_config(pat_bp_t h, int n_frames, int fmt, int* wst) {
+GatherConfig pick_config(pat_bp_t h, int n_frames, int fmt, int* wst, int max_fb) {
   const size_t limit = size_t(h->max_smem);
   if (n_frames < kStagedMinFrames && !(h->flags & PAT_FLAG_STAGED_SINGLE)) {
     // up to 3 frames: the unstaged kernels, one frame after the other (same
     // arithmetic and order as the staged kernel); units of 1 or 2 frames make
     // the staged kernel's window copies too small to pay (measured slower per
     // frame on the 3-D subject)
-    GatherConfig c = config_for(h, 1, 16, 72 * 1024, wst);
+    GatherConfig c = config_for(h, n_frames, 1, 16, 72 * 1024, wst);
     c.direct = 1;
     c.no_window = (h->flags & PAT_FLAG_NO_WINDOW) != 0;
     return c;
   }
-  for (int FB = frames_per_group(n_frames); FB >= 1; FB /= 2) {
+  for (int FB = std::min(max_fb, frames_per_unit(h, n_frames)); FB >= 1; FB /= 2) {
     const int fi = fb_index(FB);
-    GatherConfig c;
-    if (h->tuned_S[fi][fmt] > 0)
-      c = config_for(h, FB, h->tuned_S[fi][fmt], size_t(h->tuned_budget_kb[fi][fmt]) * 1024, wst);
-    else
-      c = config_for(h, FB, FB == 1 ? 16 : 8, FB == 1 ? 72 * 1024 : 100 * 1024, wst);
+    int S = h->tuned_S[fi][fmt];
+    size_t budget = size_t(h->tuned_budget_kb[fi][fmt]) * 1024;
+    if (S <= 0) default_shape(FB, limit, &S, &budget);
+    GatherConfig c = config_for(h, n_frames, FB, S, budget, wst);
     if (gather_smem_bytes(c, *wst) <= limit) return c;
-    c = config_for(h, FB, 8, limit, wst);
+    c = config_for(h, n_frames, FB, 8, limit, wst);  // longer windows: the whole SM
     if (gather_smem_bytes(c, *wst) <= limit) return c;
   }
-  return config_for(h, 1, 4, limit, wst);  // may not fit: the launch reports it
+  return config_for(h, n_frames, 1, 4, limit, wst);  // may not fit: the launch reports it
 }
 
 PreParams make_pre(pat_bp_t h, const void* sig, pat_dtype dtype, const float* scales, int n_frames,
@@ -554,11 +616,16 @@ InstDesc make_desc(pat_bp_t h, float* out, int n_frames, int FB, int wst) {
   return d;
 }
 
+int64_t unit_count(const GatherConfig& c, const InstDesc& d) {
+  const int64_t tiles = int64_t(d.n_fg) * d.n_tiles;
+  return c.FB >= 4 && !c.split ? tiles : tiles * d.n_seg;
+}
+
 int resident_ctas(const GatherConfig& c, int fmt, int wst, int n_sm) {
   // keyed by the current device too: devices of one process may differ in
   // multiprocessor count and shared memory
   struct Key {
-    int dev, n_sm, P, FB, SW, S, stages, fmt, wst, delays, wgt, direct;
+    int dev, n_sm, P, FB, SW, S, stages, fmt, wst, delays, wgt, direct, total, ring;
   };
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
@@ -569,11 +636,11 @@ int resident_ctas(const GatherConfig& c, int fmt, int wst, int n_sm) {
     const Key& k = e.first;
     if (k.dev == dev && k.n_sm == n_sm && k.P == c.P && k.FB == c.FB && k.SW == c.SW &&
         k.S == c.S && k.stages == c.stages && k.fmt == fmt && k.wst == wst &&
-        k.delays == c.delays && k.wgt == c.wgt && k.direct == c.direct)
+        k.delays == c.delays && k.wgt == c.wgt && k.direct == c.direct && k.total == c.total && k.ring == c.ring)
       return e.second;
   }
   const int r = gather_resident_ctas(c, fmt, wst, n_sm);
-  cache.push_back({Key{dev, n_sm, c.P, c.FB, c.SW, c.S, c.stages, fmt, wst, c.delays, c.wgt, c.direct}, r});
+  cache.push_back({Key{dev, n_sm, c.P, c.FB, c.SW, c.S, c.stages, fmt, wst, c.delays, c.wgt, c.direct, c.total, c.ring}, r});
   return r;
 }
 
@@ -744,7 +811,9 @@ static pat_status gather_locked(pat_bp_t h, int n_frames, float* out_dev, cudaSt
   sp.inst[0] = make_desc(h, out_dev, n_frames, c.FB, wst);
   const InstDesc& d = sp.inst[0];
   sp.n_inst = 1;
-  sp.n_units = int64_t(d.n_fg) * d.n_tiles * d.n_seg;
+  sp.n_units = unit_count(c, d);
+  sp.split = c.split;
+  sp.ring = c.ring;
   sp.S = c.S;
   sp.stages = c.stages;
   sp.Wst = wst;

@@ -43,7 +43,7 @@ struct PlanClass {
   int64_t n_units = 0;
   std::unique_ptr<PreMultiParams> pre;
   std::unique_ptr<StreamParams> gat;
-  cudaGraphNode_t pre_node = nullptr, gat_node = nullptr;
+  cudaGraphNode_t pre_node = nullptr, gat_node = nullptr, red_node = nullptr;
 };
 
 }  // namespace
@@ -76,11 +76,15 @@ struct pat_plan_s {
 namespace {
 
 int instance_fb(pat_plan_t pl, int i) {
-  return pl->fb_uniform ? pl->fb_uniform : frames_per_group(pl->frames[i]);
+  // classes of at most 8 frames per unit up to 16 frames: an instance's rows
+  // are its own, but few classes keep the launches full
+  const int F = pl->frames[i];
+  if (pl->fb_uniform) return pl->fb_uniform;
+  return F > 16 ? frames_per_group(F) : std::min(8, frames_per_group(F));
 }
 
 // Classes and launch shapes for S sensors per stage under a shared-memory
-// budget of budget_kb per CTA.
+// budget of budget_kb per CTA (0, 0: every class's own default shape).
 pat_status plan_shape(pat_plan_t pl, int S, int budget_kb) {
   pl->S = S;
   pl->budget_kb = budget_kb;
@@ -95,25 +99,55 @@ pat_status plan_shape(pat_plan_t pl, int S, int budget_kb) {
     for (size_t i = 0; i < pl->hs.size(); ++i)
       if (fbs[i] == order[c]) cls[c].idx.push_back(int(i));
   }
-  const size_t budget = std::min(size_t(budget_kb) * 1024, size_t(pl->hs[0]->max_smem));
+  const size_t limit = size_t(pl->hs[0]->max_smem);
   int64_t total_units = 0;
   for (PlanClass& k : cls) {
+    int Sk = S;
+    size_t budget = std::min(size_t(budget_kb) * 1024, limit);
+    if (S == 0) {
+      default_shape(k.FB, limit, &Sk, &budget);
+      pl->S = std::max(pl->S, Sk);
+      pl->budget_kb = std::max(pl->budget_kb, int(budget / 1024));
+    }
+    if (k.FB >= 4) Sk = std::min(Sk, 16);
     // one shape per class: the longest single window and the longest
     // S-sensor window sum of its instances bound the stages' row budget
     int wmin = 8, wfull = 8;
     for (int i : k.idx) {
       wmin = std::max(wmin, stage_window(pl->hs[i], 1));
-      wfull = std::max(wfull, stage_window(pl->hs[i], S));
+      wfull = std::max(wfull, stage_window(pl->hs[i], Sk));
     }
     GatherConfig c;
     c.P = pl->P;
     c.SW = pl->SW;
     c.delays = pl->hs[0]->delays;
     c.wgt = pl->hs[0]->wgt;
+    c.n_sm = pl->n_sm;
     c.FB = k.FB;
-    c.S = S;
+    c.S = Sk;
+    int64_t tiles = 0;
+    int n_seg = 1;
+    for (int i : k.idx) {
+      tiles += int64_t((pl->frames[i] + k.FB - 1) / k.FB) * pl->hs[i]->n_tiles;
+      n_seg = std::max(n_seg, pl->hs[i]->n_seg);
+    }
+    set_units(c, tiles, n_seg);
     int wst = wfull;
-    if (!fit_stages(c, wmin, wfull, budget, &wst))
+    bool fits = fit_stages(c, wmin, wfull, budget, &wst);
+    if (k.FB >= 4)  // smaller groups of sensors where the longest sums do not fit
+      while (!fits && c.S > 1) {
+        c.S /= 2;
+        wfull = 8;
+        for (int i : k.idx) wfull = std::max(wfull, stage_window(pl->hs[i], c.S));
+        fits = fit_stages(c, wmin, wfull, budget, &wst);
+      }
+    if (!fits && S == 0 && budget < limit) {  // a default shape too small for long windows: the whole SM
+      c.S = 4;
+      wfull = 8;
+      for (int i : k.idx) wfull = std::max(wfull, stage_window(pl->hs[i], c.S));
+      fits = fit_stages(c, wmin, wfull, limit, &wst);
+    }
+    if (!fits)
       return fail(PAT_ERR_CUDA, "stage windows do not fit in shared memory for this shape");
     k.cfg = c;
     k.wst = wst;
@@ -134,7 +168,7 @@ pat_status plan_shape(pat_plan_t pl, int S, int budget_kb) {
       const int F = pl->frames[k.idx[j]];
       sp.inst[j] = make_desc(h, nullptr, F, k.FB, wst);
       sp.inst[j].unit_begin = units;
-      units += int64_t(sp.inst[j].n_fg) * sp.inst[j].n_tiles * sp.inst[j].n_seg;
+      units += unit_count(c, sp.inst[j]);
       pm.inst[j] = make_pre(h, nullptr, pl->dtype, nullptr, F, k.FB);
       pm.cta_begin[j] = ctas;
       ctas += int64_t(h->ns) * sp.inst[j].n_fg;
@@ -150,6 +184,8 @@ pat_status plan_shape(pat_plan_t pl, int S, int budget_kb) {
     sp.S = c.S;
     sp.stages = c.stages;
     sp.Wst = wst;
+    sp.split = c.split;
+    sp.ring = c.ring;
     sp.status = pl->d_status;
     sp.sched = pl->d_sched;
     sp.timeout_ns = 2000000000ull;
@@ -199,7 +235,7 @@ void drop_graph(pat_plan_t pl) {
   if (pl->graph) cudaGraphDestroy(pl->graph);
   pl->exec = nullptr;
   pl->graph = nullptr;
-  for (PlanClass& k : pl->cls) k.pre_node = k.gat_node = nullptr;
+  for (PlanClass& k : pl->cls) k.pre_node = k.gat_node = k.red_node = nullptr;
 }
 
 // Point every descriptor at the handles' current buffers: a handle's own
@@ -268,12 +304,15 @@ pat_status capture(pat_plan_t pl) {
       if (kp.func == gather_kernel_func(k.cfg, pl->fmt) &&
           std::memcmp(kp.kernelParams[0], k.gat.get(), sizeof(StreamParams)) == 0)
         k.gat_node = nd;
+      if (k.FB >= 4 && kp.func == rows_reduce_func(k.FB) &&
+          std::memcmp(kp.kernelParams[0], k.gat.get(), sizeof(StreamParams)) == 0)
+        k.red_node = nd;
     }
   }
   for (PlanClass& k : pl->cls)
-    if (k.n_units > 0 && (!k.pre_node || !k.gat_node)) {
+    if (k.n_units > 0 && (!k.pre_node || !k.gat_node || (!k.red_node && rows_needs_reduce(*k.gat)))) {
       cudaGraphDestroy(g);
-      for (PlanClass& c : pl->cls) c.pre_node = c.gat_node = nullptr;
+      for (PlanClass& c : pl->cls) c.pre_node = c.gat_node = c.red_node = nullptr;
       return fail(PAT_ERR_CUDA, "captured graph lacks the expected kernels");
     }
   pl->graph = g;
@@ -295,6 +334,12 @@ pat_status refresh_graph(pat_plan_t pl) {
     kp.kernelParams = gat_args;
     kp.extra = nullptr;
     PAT_CUDA(cudaGraphExecKernelNodeSetParams(pl->exec, k.gat_node, &kp));
+    if (!k.red_node) continue;
+    void* red_args[2] = {k.gat.get(), &k.cfg.P};
+    PAT_CUDA(cudaGraphKernelNodeGetParams(k.red_node, &kp));
+    kp.kernelParams = red_args;
+    kp.extra = nullptr;
+    PAT_CUDA(cudaGraphExecKernelNodeSetParams(pl->exec, k.red_node, &kp));
   }
   return PAT_OK;
 }
@@ -355,7 +400,7 @@ pat_status autotune(pat_plan_t pl, const void* const* sig, const float* const* s
       return s;
     }
   }
-  const int Ss[4] = {4, 8, 16, 32};
+  const int Ss[5] = {0, 4, 8, 16, 32};  // 0: the default shapes of the classes
   const int budgets[4] = {55, 72, 110, pl->hs[0]->max_smem / 1024};
   cudaEvent_t e0, e1;
   PAT_CUDA(cudaEventCreate(&e0));
@@ -365,8 +410,8 @@ pat_status autotune(pat_plan_t pl, const void* const* sig, const float* const* s
   pat_status st_all = PAT_OK;
   for (int S : Ss)
     for (int b : budgets) {
-      if (S == 4 && b != budgets[3]) continue;  // 4 sensors per stage only as a last resort
-      pat_status s = plan_shape(pl, S, b);
+      if (S == 0 && b != budgets[0]) continue;
+      pat_status s = plan_shape(pl, S, S ? b : 0);
       if (s != PAT_OK) continue;
       if ((s = refresh_buffers(pl)) != PAT_OK) {
         st_all = s;
@@ -391,7 +436,7 @@ pat_status autotune(pat_plan_t pl, const void* const* sig, const float* const* s
       if (ms < best) {
         best = ms;
         bs = S;
-        bb = b;
+        bb = S ? b : 0;
       }
     }
   cudaEventDestroy(e0);
@@ -455,11 +500,11 @@ static pat_status plan_new(const pat_bp_t* handles, const int* n_frames, int n, 
     pl->d_status = handles[0]->d_status;
     pl->d_sched = handles[0]->d_sched;
   }
-  // default shape: 8 sensors per stage in 100 KB; if the stage windows do not
-  // fit, the device's limit, then 4 sensors per stage
+  // the default shapes; if the stage windows do not fit, 8 and then 4 sensors
+  // per stage in the device's limit
   pat_status st = PAT_ERR_CUDA;
   const int limit_kb = handles[0]->max_smem / 1024;
-  const int tries[3][2] = {{8, 100}, {8, limit_kb}, {4, limit_kb}};
+  const int tries[3][2] = {{0, 0}, {8, limit_kb}, {4, limit_kb}};
   for (const auto& t : tries) {
     st = plan_shape(pl.get(), t[0], t[1]);
     if (st == PAT_OK) break;
@@ -606,7 +651,9 @@ extern "C" pat_status pat_bp_autotune(pat_bp_t h, const void* signals_dev, pat_d
   if (!h) return fail(PAT_ERR_INVALID, "NULL handle");
   std::lock_guard<std::mutex> lk(h->mu);
   pat_plan_t pl = nullptr;
-  pat_status st = plan_new(&h, &n_frames, 1, dtype, 0, false, frames_per_group(n_frames), &pl);
+  pat_status st = plan_new(&h, &n_frames, 1, dtype, 0, false,
+                           n_frames < kStagedMinFrames ? frames_per_group(n_frames) : frames_per_unit(h, n_frames),
+                           &pl);
   if (st != PAT_OK) return st;
   const void* sig[1] = {signals_dev};
   const float* sc[1] = {scales_dev};
