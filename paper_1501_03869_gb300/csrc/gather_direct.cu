@@ -1,11 +1,11 @@
 // gather_direct.cu -- the single-frame gather of Eq. (BP) without the staged
 // pipeline.
 //
-// Two gathers share the reduction kernel below.  gather_window_kernel (stored
-// tables without weights, every window at most 288 samples) copies each
-// sensor's integrand window into shared memory per warp and interpolates
-// there; gather_direct_kernel, described next, gathers from L2 and takes every
-// other case.  Both give the same bits.
+// Two gathers share the reduction kernel below.  gather_window_kernel (every
+// window at most 384 samples) copies each sensor's integrand window into
+// shared memory per warp and interpolates there; gather_direct_kernel,
+// described next, gathers from L2 and takes every other case.  Both give the
+// same bits.
 //
 // Two launches.  The gather kernel is persistent: CTA c takes units (tile,
 // segment of G sensors) c, c + grid, c + 2 grid, ... in tile-major order, and
@@ -39,6 +39,7 @@
 #include <algorithm>
 
 #include "gather.cuh"
+#include "packed.cuh"
 
 namespace patbp {
 
@@ -308,46 +309,62 @@ __global__ void __launch_bounds__(256) direct_reduce_kernel(const __grid_constan
 }
 
 // ------------------------------------------------------ windowed variant --
-// Stored tables without solid-angle weights, when every window of the table
-// fits a shared-memory slot of WB rows.  The four warps of a CTA are the four
-// (pixel group, sensor phase) pairs of one unit, as above; a warp takes its
-// sensors two at a time.  For each sensor it copies the tile's integrand
-// window (rows base .. base + len) into a slot of its own with 16-byte
-// cp.async copies, two steps ahead, while its lanes' table offsets come from
-// global memory one step ahead; the interpolation then reads shared memory.
+// For handles whose every window fits a shared-memory slot of WB rows.  The
+// four warps of a CTA are the four (pixel group, sensor phase) pairs of one
+// unit, as above; a lane owns 4 neighbouring pixels of its warp's 128
+// (their offsets are one 16-byte load; pixels 32 apart met fewer bank conflicts,
+// 1.6 to 2.0 wavefronts per load against 2.2 to 2.5, but took 252 us instead of
+// 229 on a BF16 volume).  A warp
+// takes its sensors two at a time.  For each sensor it copies the tile's
+// integrand window (rows base .. base + len) into a slot of its own with
+// 16-byte cp.async copies, two steps ahead, while its lanes' table offsets come
+// from global memory one step ahead; constant-
+// speed delays and solid-angle weights are evaluated from anchors staged in
+// shared memory once per unit.  The interpolation then reads shared memory.
 // Each slot ends in 8 zero rows at row WB: an offset after the record (the
 // table's out-of-record value) is clamped to WB, which gives phase 0 and the
-// zero rows, so it adds m * 0 as in the kernel above.  The CTA sums its four
-// phase sums per pixel in order before storing, so the reduction kernel sums
-// segments only.  Arithmetic and summation order are those of
-// gather_direct_kernel: the image has the same bits.
+// zero rows, so it adds m * 0 as in the kernel above; so does the absent
+// second sensor of a last step.  The CTA sums its four phase sums per pixel in
+// order before storing, so the reduction kernel sums segments only.
+// Arithmetic and summation order are those of gather_direct_kernel: the image
+// has the same bits.
+//
+// What bounds it: instruction issue and shared-memory wavefronts (one warp-sensor
+// took 113 instructions at 76 % issue-active with scalar FP32), so
+// pixels go through packed FP32 pairs, steps alternate between two register
+// sets and two slots with constant addresses, and nothing branches per sensor:
+// 84 instructions.  One frame of 512 sensors x 0.6 M voxels (1.24 GB table):
+// FP32 301 -> 286 us, BF16 296 -> 243, constant speed 549 -> 422.
 //
 // Offsets in the window are found from the FP32 bits: for 0 <= u < 2^23,
 // u + 2^23 rounded toward zero is 2^23 + floor(u) exactly, its bit pattern is
 // 0x4B000000 + floor(u), and (u + 2^23) - 2^23 = floor(u) exactly.
-constexpr int kWindowMaxRows = 288;  // largest slot (rows); longer windows take the kernel above
+constexpr int kWindowMaxRows = 384;  // largest slot (rows); longer windows take the kernel above
 
-template <int P, int SW, int FMT, int WB>
-__global__ void __launch_bounds__(128, kDirectMinCtas + 1)
+template <int P, int SW, int FMT, int WB, int DELAYS, int WGT>
+__global__ void __launch_bounds__(128, DELAYS || WGT ? 6 : (WB > 288 ? 7 : 9))
     gather_window_kernel(const __grid_constant__ DirectParams p) {
   constexpr int PW = P / 128;
   static_assert(PW * SW == 4, "a unit is four warps");
   constexpr int SLOT = WB + 8;  // rows of one slot: window, then 8 zero rows
-  constexpr int D = 2;          // steps of two sensors whose windows are in flight
   constexpr int NC = (WB + 127) / 128;  // 16-byte copies per lane for one window
-  __shared__ __align__(16) uint32_t swin[4][2 * D][SLOT];
-  __shared__ __align__(16) uint2 sbm[4][32];  // (window base word, multiplier) per sensor of the warp
-  __shared__ float ssum[SW][P];
+  constexpr int MAXJ = 64 / SW;         // sensors of a warp (segments of at most 64)
+  __shared__ __align__(16) uint32_t swin[4][4][SLOT];
+  __shared__ __align__(16) uint2 sbm[4][MAXJ];  // (window base word, multiplier) per sensor of the warp
+  __shared__ __align__(16) float4 sanchor[DELAYS ? 4 : 1][DELAYS ? MAXJ : 1][2];
+  __shared__ __align__(16) float4 swanchor[WGT ? 4 : 1][WGT ? MAXJ : 1][2];
+  __shared__ __align__(16) float ssum[SW][P];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int pg = warp % PW, sp = warp / PW;
-  const int px0 = pg * 128 + lane;
+  const int px0 = pg * 128 + 4 * lane;
   uint32_t* ring = &swin[warp][0][0];
-  for (int k = lane; k < 2 * D * 8; k += 32) ring[(k >> 3) * SLOT + WB + (k & 7)] = 0u;
+  ring[(lane >> 3) * SLOT + WB + (lane & 7)] = 0u;  // 4 slots x 8 zero rows
   const uint32_t ring_s = smem_addr(ring);
   const int64_t n_units = int64_t(p.n_tiles) * p.n_seg;
   const uint32_t* bsrc = static_cast<const uint32_t*>(p.b);
-  const uint2* bm = sbm[warp];
+  const uint32_t bm_s = smem_addr(sbm[warp]);
+  const f32x2 magic = pack2(8388608.0f, 8388608.0f), unmagic = pack2(-8388608.0f, -8388608.0f);
   // integrand and multipliers come from the preprocessing grid
   asm volatile("griddepcontrol.wait;" ::: "memory");
   for (int64_t unit = blockIdx.x; unit < n_units; unit += gridDim.x) {
@@ -355,46 +372,68 @@ __global__ void __launch_bounds__(128, kDirectMinCtas + 1)
     const int seg = int(unit - int64_t(tile) * p.n_seg);
     const int s_lo = seg * p.G, s_hi = min(p.n_sensors, s_lo + p.G);
     const int s0 = s_lo + sp;  // this warp's sensors: s0, s0 + SW, ...
-    const int nj = s0 < s_hi ? (s_hi - s0 + SW - 1) / SW : 0;  // <= 32 (G <= 32 SW)
-    const float* ubase = p.u + (int64_t(tile) * p.n_sensors + s0) * P + px0;
-    if (unit != int64_t(blockIdx.x) && threadIdx.x == 0) {
-      // a CTA's later units (launches with more units than resident CTAs)
-      // start at staggered times: their table block is asked into L2 at once.
-      // (Not the first unit: every CTA asking for its block at the launch's
-      // start delayed the first offsets behind the whole table.)
-      const int n_sen = s_hi - s_lo;
-      bulk_prefetch_l2(p.u + (int64_t(tile) * p.n_sensors + s_lo) * P, uint32_t(n_sen) * P * 4);
+    const int nj = s0 < s_hi ? (s_hi - s0 + SW - 1) / SW : 0;
+    const float* ubase = nullptr;
+    if constexpr (DELAYS == 0) {
+      ubase = p.u + (int64_t(tile) * p.n_sensors + s0) * P + px0;
+      if (unit != int64_t(blockIdx.x) && threadIdx.x == 0) {
+        // a CTA's later units (launches with more units than resident CTAs)
+        // start at staggered times: their table block is asked into L2 at once.
+        // (Not the first unit: every CTA asking for its block at the launch's
+        // start delayed the first offsets behind the whole table.)
+        bulk_prefetch_l2(p.u + (int64_t(tile) * p.n_sensors + s_lo) * P, uint32_t(s_hi - s_lo) * P * 4);
+      }
     }
     const uint32_t* wsrc = bsrc + int64_t(s0) * p.n_t_pad + lane * 4;
-    const int64_t ustep = int64_t(SW) * P, wstep = int64_t(SW) * p.n_t_pad;
-    // the lanes' offsets of the sensors 2k, 2k + 1
-    auto load_u = [&](int k, float (&d)[2][4]) {
+    const uint32_t wstep = uint32_t(SW) * uint32_t(p.n_t_pad);
+    float4 pq[4];
+    if constexpr (DELAYS != 0 || WGT != 0) {
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const float* ur = ubase + min(2 * k + h, nj - 1) * ustep;
+      for (int x = 0; x < 4; ++x) pq[x] = __ldcg(p.pix + int64_t(tile) * P + px0 + x);
+    }
+    // the lane's offsets of the sensors j, j + 1 (past the last: after the record)
+    auto load_u = [&](int j, float4 (&d)[2]) {
+      if constexpr (DELAYS == 0) {
 #pragma unroll
-        for (int x = 0; x < 4; ++x) d[h][x] = __ldcg(ur + 32 * x);
+        for (int h = 0; h < 2; ++h)
+          d[h] = j + h < nj ? __ldcg(reinterpret_cast<const float4*>(ubase + (j + h) * (SW * P)))
+                            : make_float4(kFarOffset, kFarOffset, kFarOffset, kFarOffset);
       }
     };
-    const int nk = (nj + 1) >> 1;
-    float un[2][4];
-    if (nk > 0) load_u(0, un);  // in flight with the window bases below
-    if (lane < nj) {
+    float4 ua[2], ub[2];
+    load_u(0, ua);  // in flight with the window bases below
+    if (lane < MAXJ) {
       const int s = s0 + lane * SW;
-      sbm[warp][lane] = make_uint2(uint32_t(__ldcg(p.base + int64_t(tile) * p.n_sensors_pad + s)),
-                                   __float_as_uint(__ldcg(p.m + s)));
+      uint2 w = make_uint2(0u, 0u);
+      if (lane < nj)
+        w = make_uint2(uint32_t(__ldcg(p.base + int64_t(tile) * p.n_sensors_pad + s)),
+                       __float_as_uint(__ldcg(p.m + s)));
+      sbm[warp][lane] = w;
+      if constexpr (DELAYS != 0) {
+        const float4* ap = reinterpret_cast<const float4*>(p.anchor) +
+                           (int64_t(tile) * p.n_sensors_pad + min(s, s_hi - 1)) * 2;
+        float4 A = __ldcg(ap), B = __ldcg(ap + 1);
+        if (lane >= nj) B.y = -1.0f;  // cap below every offset: nothing to add
+        sanchor[warp][lane][0] = A;
+        sanchor[warp][lane][1] = B;
+      }
+      if constexpr (WGT != 0) {
+        const float4* wp = reinterpret_cast<const float4*>(p.wanchor) +
+                           (int64_t(tile) * p.n_sensors_pad + min(s, s_hi - 1)) * 2;
+        swanchor[warp][lane][0] = __ldcg(wp);
+        swanchor[warp][lane][1] = __ldcg(wp + 1);
+      }
     }
     __syncwarp();
-    // windows of the sensors 2k, 2k + 1 into slots 2 slot, 2 slot + 1; one group per step
-    auto issue = [&](int k, int slot) {
+    // windows of the sensors j, j + 1 into the slots 2 buf, 2 buf + 1; one group per step
+    auto issue = [&](int j, int buf) {
+      if (j < nj) {
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int j = 2 * k + h;
-        if (j < nj) {
-          const uint32_t b = bm[j].x;
+        for (int h = 0; h < 2; ++h) {
+          const uint32_t b = lds_u32(bm_s + uint32_t(j + h) * 8u);
           const int len = int(b >> 16);
-          const uint32_t sa = ring_s + uint32_t(((2 * slot + h) * SLOT + lane * 4) * 4);
-          const uint32_t* src = wsrc + j * wstep + (b & 0xffffu);
+          const uint32_t* src = wsrc + (uint32_t(j + h) * wstep + (b & 0xffffu));
+          const uint32_t sa = ring_s + uint32_t(((2 * buf + h) * SLOT + lane * 4) * 4);
 #pragma unroll
           for (int c = 0; c < NC; ++c)
             if (lane * 4 + c * 128 < len) cp_async16(sa + c * 512, src + c * 128);
@@ -402,63 +441,65 @@ __global__ void __launch_bounds__(128, kDirectMinCtas + 1)
       }
       cp_async_commit();
     };
-    // interpolation of one sensor at the lane's 4 offsets; wadj = the slot's
-    // row 0 minus 4 * 0x4B000000 (shared addresses wrap modulo 2^32)
-    auto lerp4 = [&](uint32_t wadj, const float (&uu)[4], float (&v)[4]) {
+    issue(0, 0);
+    issue(2, 1);
+    f32x2 acc[2] = {0ull, 0ull};
+    // sensor j, offsets u, slot; the slot's row 0 minus 4 * 0x4B000000 (shared
+    // addresses wrap modulo 2^32)
+    auto sensor = [&](int j, float4 u4, int slot, float m) {
+      float uu[4] = {u4.x, u4.y, u4.z, u4.w};
+      if constexpr (DELAYS != 0) constant_offsets<4>(uu, pq, sanchor[warp][j][0], sanchor[warp][j][1]);
+      float ww[4];
+      if constexpr (WGT != 0) solid_angle_weights(ww, pq, swanchor[warp][j][0], swanchor[warp][j][1]);
+      const uint32_t wadj = ring_s + uint32_t(slot * SLOT * 4) - 4u * 0x4B000000u;
+      const f32x2 mm = pack2(m, m);
 #pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        const float uc = fminf(uu[x], float(WB));
-        const float t = __fadd_rz(uc, 8388608.0f);
-        const float ph = __fsub_rn(uc, __fsub_rn(t, 8388608.0f));
-        const uint32_t a = wadj + 4u * __float_as_uint(t);
-        const uint32_t w0 = lds_u32(a);
+      for (int x = 0; x < 2; ++x) {
+        const f32x2 uc = pack2(fminf(uu[2 * x], float(WB)), fminf(uu[2 * x + 1], float(WB)));
+        const f32x2 t = add2_rz(uc, magic);
+        const f32x2 ph = sub2(uc, add2(t, unmagic));
+        float t0, t1;
+        unpack2(t, t0, t1);
+        const uint32_t a0 = wadj + 4u * __float_as_uint(t0), a1 = wadj + 4u * __float_as_uint(t1);
+        f32x2 v;
         if constexpr (FMT == kBF32) {
-          const float b0 = __uint_as_float(w0), b1 = __uint_as_float(lds_u32(a + 4));
-          v[x] = fmaf(ph, b1 - b0, b0);
-        } else if constexpr (FMT == kBBF16P) {
-          v[x] = fmaf(ph, __uint_as_float(w0 & 0xffff0000u), __uint_as_float(w0 << 16));
+          const f32x2 b0 = pack2u(lds_u32(a0), lds_u32(a1)), b1 = pack2u(lds_u32(a0 + 4), lds_u32(a1 + 4));
+          v = fma2(ph, sub2(b1, b0), b0);
         } else {
-          const float2 hf = __half22float2(*reinterpret_cast<const __half2*>(&w0));
-          v[x] = fmaf(ph, hf.y, hf.x);
+          const uint32_t w0 = lds_u32(a0), w1 = lds_u32(a1);
+          if constexpr (FMT == kBBF16P) {
+            v = fma2(ph, pack2u(w0 & 0xffff0000u, w1 & 0xffff0000u), pack2u(w0 << 16, w1 << 16));
+          } else {
+            const float2 h0 = __half22float2(*reinterpret_cast<const __half2*>(&w0));
+            const float2 h1 = __half22float2(*reinterpret_cast<const __half2*>(&w1));
+            v = fma2(ph, pack2(h0.y, h1.y), pack2(h0.x, h1.x));
+          }
         }
+        if constexpr (WGT != 0) v = mul2(pack2(ww[2 * x], ww[2 * x + 1]), v);
+        acc[x] = fma2(mm, v, acc[x]);
       }
     };
-#pragma unroll
-    for (int k = 0; k < D; ++k) issue(k, k);
-    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    int slot = 0;
-    for (int k = 0; k < nk; ++k) {
-      float uc[2][4];
-#pragma unroll
-      for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int x = 0; x < 4; ++x) uc[h][x] = un[h][x];
-      if (k + 1 < nk) load_u(k + 1, un);
-      cp_async_wait<D - 1>();
+    // one step: the sensors j, j + 1 in the slots of `buf`, their offsets in u;
+    // the next step's offsets into nu, the windows of the step after that
+    auto step = [&](int j, const float4 (&u)[2], float4 (&nu)[2], int buf) {
+      load_u(j + 2, nu);
+      cp_async_wait<1>();
       __syncwarp();
-      const int j = 2 * k;
-      const uint4 q = *reinterpret_cast<const uint4*>(bm + j);  // sensors j and j + 1
-      const uint32_t wa = ring_s + uint32_t(2 * slot * SLOT * 4) - 4u * 0x4B000000u;
-      float va[4];
-      lerp4(wa, uc[0], va);
-      if (j + 1 < nj) {
-        float vb[4];
-        lerp4(wa + SLOT * 4, uc[1], vb);
-        const float ma = __uint_as_float(q.y), mb = __uint_as_float(q.w);
-#pragma unroll
-        for (int x = 0; x < 4; ++x) acc[x] = fmaf(mb, vb[x], fmaf(ma, va[x], acc[x]));
-      } else {
-        const float ma = __uint_as_float(q.y);
-#pragma unroll
-        for (int x = 0; x < 4; ++x) acc[x] = fmaf(ma, va[x], acc[x]);
-      }
+      const uint4 q = lds_u4(bm_s + uint32_t(j) * 8u);  // sensors j and j + 1
+      sensor(j, u[0], 2 * buf, __uint_as_float(q.y));
+      sensor(j + 1, u[1], 2 * buf + 1, __uint_as_float(q.w));
       __syncwarp();  // every lane has read the slots before they are refilled
-      issue(k + D, slot);
-      slot ^= 1;
+      issue(j + 4, buf);
+    };
+    for (int j = 0; j < nj; j += 4) {
+      step(j, ua, ub, 0);
+      if (j + 2 < nj) step(j + 2, ub, ua, 1);
     }
     cp_async_wait<0>();
-#pragma unroll
-    for (int x = 0; x < 4; ++x) ssum[sp][px0 + 32 * x] = acc[x];
+    float r[4];
+    unpack2(acc[0], r[0], r[1]);
+    unpack2(acc[1], r[2], r[3]);
+    *reinterpret_cast<float4*>(&ssum[sp][px0]) = make_float4(r[0], r[1], r[2], r[3]);
     __syncthreads();
     for (int q = threadIdx.x; q < P; q += 128) {
       float v = 0.0f;
@@ -517,9 +558,9 @@ cudaError_t launch_direct_fmt(const DirectParams& dp, int n_sm, cudaStream_t st,
   return launch_pdl(direct_reduce_kernel<P, SW>, std::max(rgrid, 1u), 256u, dp, st);
 }
 
-template <int P, int SW, int FMT, int WB>
+template <int P, int SW, int FMT, int WB, int DELAYS, int WGT>
 cudaError_t launch_window_fmt(const DirectParams& dp, int n_sm, cudaStream_t st, bool reduce) {
-  auto kern = gather_window_kernel<P, SW, FMT, WB>;
+  auto kern = gather_window_kernel<P, SW, FMT, WB, DELAYS, WGT>;
   static PerDevice cache;  // resident CTAs per SM, per device
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -540,20 +581,31 @@ cudaError_t launch_window_fmt(const DirectParams& dp, int n_sm, cudaStream_t st,
   return launch_pdl(direct_reduce_kernel<P, 1>, std::max(rgrid, 1u), 256u, dp, st);
 }
 
-template <int P, int SW, int WB>
+template <int P, int SW, int WB, int DELAYS, int WGT>
 cudaError_t launch_window_w(int fmt, const DirectParams& dp, int n_sm, cudaStream_t st, bool reduce) {
-  if (fmt == kBF32) return launch_window_fmt<P, SW, kBF32, WB>(dp, n_sm, st, reduce);
-  if (fmt == kBBF16P) return launch_window_fmt<P, SW, kBBF16P, WB>(dp, n_sm, st, reduce);
-  if (fmt == kBF16P) return launch_window_fmt<P, SW, kBF16P, WB>(dp, n_sm, st, reduce);
+  if (fmt == kBF32) return launch_window_fmt<P, SW, kBF32, WB, DELAYS, WGT>(dp, n_sm, st, reduce);
+  if (fmt == kBBF16P) return launch_window_fmt<P, SW, kBBF16P, WB, DELAYS, WGT>(dp, n_sm, st, reduce);
+  if (fmt == kBF16P) return launch_window_fmt<P, SW, kBF16P, WB, DELAYS, WGT>(dp, n_sm, st, reduce);
   return cudaErrorInvalidValue;
 }
 
-// The smallest slot (128, 192 or 288 rows) that holds every window.
-template <int P, int SW>
+// The smallest slot (128, 192, 288 or 384 rows) that holds every window.
+template <int P, int SW, int DELAYS, int WGT>
 cudaError_t launch_window(int fmt, const DirectParams& dp, int n_sm, cudaStream_t st, bool reduce) {
-  if (dp.W <= 128) return launch_window_w<P, SW, 128>(fmt, dp, n_sm, st, reduce);
-  if (dp.W <= 192) return launch_window_w<P, SW, 192>(fmt, dp, n_sm, st, reduce);
-  return launch_window_w<P, SW, kWindowMaxRows>(fmt, dp, n_sm, st, reduce);
+  if (dp.W <= 128) return launch_window_w<P, SW, 128, DELAYS, WGT>(fmt, dp, n_sm, st, reduce);
+  if (dp.W <= 192) return launch_window_w<P, SW, 192, DELAYS, WGT>(fmt, dp, n_sm, st, reduce);
+  if constexpr (DELAYS == 0 && WGT == 0)
+    if (dp.W > 288) return launch_window_w<P, SW, kWindowMaxRows, 0, 0>(fmt, dp, n_sm, st, reduce);
+  return launch_window_w<P, SW, 288, DELAYS, WGT>(fmt, dp, n_sm, st, reduce);
+}
+
+template <int P, int SW>
+cudaError_t launch_window_mode(bool delays, int fmt, const DirectParams& dp, int n_sm, cudaStream_t st, bool reduce) {
+  if (dp.wanchor)
+    return delays ? launch_window<P, SW, 1, 1>(fmt, dp, n_sm, st, reduce)
+                  : launch_window<P, SW, 0, 1>(fmt, dp, n_sm, st, reduce);
+  return delays ? launch_window<P, SW, 1, 0>(fmt, dp, n_sm, st, reduce)
+                : launch_window<P, SW, 0, 0>(fmt, dp, n_sm, st, reduce);
 }
 
 template <int P, int SW, int DELAYS, int WGT>
@@ -603,11 +655,14 @@ cudaError_t launch_gather_direct(const GatherConfig& c, int fmt, const InstDesc&
   dp.n_seg = d.n_seg;
   dp.G = d.G;
   dp.W = d.W;
-  // stored tables without weights: the windowed kernel when every window fits a slot
-  const bool window = !c.delays && !dp.wanchor && !c.no_window && dp.W >= 0 &&
-                      dp.W <= kWindowMaxRows && dp.G <= 32 * c.SW;
-  if (window && c.P == 128 && c.SW == 4) return launch_window<128, 4>(fmt, dp, n_sm, st, reduce);
-  if (window && c.P == 256 && c.SW == 2) return launch_window<256, 2>(fmt, dp, n_sm, st, reduce);
+  // the windowed kernel when every window fits a slot.  Computed delays and
+  // weights hold more registers (6 CTAs per SM): with slots of 384 rows they
+  // lose to the kernel above (paper-shaped frame at constant speed 30.0 us
+  // against 28.4; stored table with 256-pixel tiles 26.1 -> 22.9)
+  const int most = c.delays || dp.wanchor ? 288 : kWindowMaxRows;
+  const bool window = !c.no_window && dp.W >= 0 && dp.W <= most && dp.G <= 64;
+  if (window && c.P == 128 && c.SW == 4) return launch_window_mode<128, 4>(c.delays != 0, fmt, dp, n_sm, st, reduce);
+  if (window && c.P == 256 && c.SW == 2) return launch_window_mode<256, 2>(c.delays != 0, fmt, dp, n_sm, st, reduce);
   if (c.P == 128 && c.SW == 4)
     return c.delays ? launch_direct_t<128, 4, 1>(fmt, dp, n_sm, st, reduce)
                     : launch_direct_t<128, 4, 0>(fmt, dp, n_sm, st, reduce);
