@@ -260,6 +260,14 @@ __global__ void __launch_bounds__(32 * (P / 128) * SW, kDirectMinCtas)
   if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// Clears the image outside the mask (CTAs of a grid share the runs).
+__device__ __forceinline__ void clear_outside(const DirectParams& p) {
+  for (int r = blockIdx.x; r < p.n_zero_runs; r += gridDim.x) {
+    const int st0 = p.zero_runs[2 * r], len = p.zero_runs[2 * r + 1];
+    for (int i = threadIdx.x; i < len; i += blockDim.x) p.out[st0 + i] = 0.0f;
+  }
+}
+
 // Sum of every pixel over phases (in order) and segments (in order), written
 // to its place in the image (SW = 1: the part buffer holds segment sums); also clears the image outside the mask.  The
 // loads of 8 segments are issued before their sums, so a pixel costs about
@@ -267,10 +275,7 @@ __global__ void __launch_bounds__(32 * (P / 128) * SW, kDirectMinCtas)
 template <int P, int SW>
 __global__ void __launch_bounds__(256) direct_reduce_kernel(const __grid_constant__ DirectParams p) {
   constexpr int K = 8;
-  for (int64_t r = blockIdx.x; r < p.n_zero_runs; r += gridDim.x) {
-    const int st0 = p.zero_runs[2 * r], len = p.zero_runs[2 * r + 1];
-    for (int i2 = threadIdx.x; i2 < len; i2 += blockDim.x) p.out[st0 + i2] = 0.0f;
-  }
+  clear_outside(p);
   asm volatile("griddepcontrol.wait;" ::: "memory");
   // the kernels before this one are complete: their status is final
   if (p.host_status && blockIdx.x == 0 && threadIdx.x == 0) *p.host_status = __ldcg(p.status);
@@ -325,7 +330,9 @@ __global__ void __launch_bounds__(256) direct_reduce_kernel(const __grid_constan
 // table's out-of-record value) is clamped to WB, which gives phase 0 and the
 // zero rows, so it adds m * 0 as in the kernel above; so does the absent
 // second sensor of a last step.  The CTA sums its four phase sums per pixel in
-// order before storing, so the reduction kernel sums segments only.
+// order before storing, so the reduction kernel sums segments only; with one
+// segment per tile (at most 64 sensors) the sums go to the image and there is no
+// reduction launch.
 // Arithmetic and summation order are those of gather_direct_kernel: the image
 // has the same bits.
 //
@@ -365,8 +372,12 @@ __global__ void __launch_bounds__(128, DELAYS || WGT ? 6 : (WB > 288 ? 7 : 9))
   const uint32_t* bsrc = static_cast<const uint32_t*>(p.b);
   const uint32_t bm_s = smem_addr(sbm[warp]);
   const f32x2 magic = pack2(8388608.0f, 8388608.0f), unmagic = pack2(-8388608.0f, -8388608.0f);
+  // one segment per tile: its sums are the image, and no reduction follows
+  const bool final = p.out && p.n_seg == 1;
+  if (final) clear_outside(p);
   // integrand and multipliers come from the preprocessing grid
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (final && p.host_status && blockIdx.x == 0 && threadIdx.x == 0) *p.host_status = __ldcg(p.status);
   for (int64_t unit = blockIdx.x; unit < n_units; unit += gridDim.x) {
     const int tile = int(unit / p.n_seg);
     const int seg = int(unit - int64_t(tile) * p.n_seg);
@@ -505,7 +516,12 @@ __global__ void __launch_bounds__(128, DELAYS || WGT ? 6 : (WB > 288 ? 7 : 9))
       float v = 0.0f;
 #pragma unroll
       for (int ph = 0; ph < SW; ++ph) v += ssum[ph][q];
-      p.part[(int64_t(tile) * p.n_seg + seg) * P + q] = v;
+      if (final) {
+        const int o = __ldcg(p.slot + int64_t(tile) * P + q);
+        if (o >= 0) p.out[o] = v;
+      } else {
+        p.part[(int64_t(tile) * p.n_seg + seg) * P + q] = v;
+      }
     }
     __syncthreads();
   }
@@ -575,7 +591,7 @@ cudaError_t launch_window_fmt(const DirectParams& dp, int n_sm, cudaStream_t st,
   const int64_t n_units = int64_t(dp.n_tiles) * dp.n_seg;
   const unsigned grid = unsigned(std::min<int64_t>(n_units, int64_t(cache.per_sm[dev]) * n_sm));
   e = launch_pdl(kern, grid, 128u, dp, st);
-  if (e != cudaSuccess || !reduce) return e;
+  if (e != cudaSuccess || !reduce || dp.n_seg == 1) return e;  // one segment: the gather wrote the image
   const int64_t n = int64_t(dp.n_tiles) * P;
   const unsigned rgrid = unsigned(std::min<int64_t>((n + 255) / 256, int64_t(n_sm) * 8));
   return launch_pdl(direct_reduce_kernel<P, 1>, std::max(rgrid, 1u), 256u, dp, st);
