@@ -28,24 +28,33 @@ __all__ = ["BP", "Plan", "Server", "PatError", "fmm_host", "fmm_gpu", "table_hos
 DTYPES = {"f32": _lib.PAT_F32, "bf16": _lib.PAT_BF16, "f16": _lib.PAT_F16}
 
 
+_torch_module = None
+_dtype_codes = {}
+
+
 def _torch():
-    import torch
-    return torch
+    """torch, imported at the first call that needs it."""
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _dtype_codes.update({torch.float32: _lib.PAT_F32, torch.bfloat16: _lib.PAT_BF16,
+                             torch.float16: _lib.PAT_F16})
+        _torch_module = torch
+    return _torch_module
 
 
 def _dtype_code(t):
-    torch = _torch()
-    m = {torch.float32: _lib.PAT_F32, torch.bfloat16: _lib.PAT_BF16, torch.float16: _lib.PAT_F16}
-    if t.dtype not in m:
+    _torch()
+    code = _dtype_codes.get(t.dtype)
+    if code is None:
         raise TypeError(f"signals must be float32, bfloat16 or float16, not {t.dtype}")
-    return m[t.dtype]
+    return code
 
 
 def _stream_ptr(stream):
-    torch = _torch()
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        stream = _torch().cuda.current_stream()
+    return stream.cuda_stream
 
 
 class BP:
@@ -112,6 +121,7 @@ class BP:
         inf = _lib.PatInfo()
         _lib.check(self._lib.pat_bp_info(self._h, ctypes.byref(inf)), "pat_bp_info")
         self.info = {k: getattr(inf, k) for k, _ in _lib.PatInfo._fields_}
+        self._frame_numel = int(inf.n_pix if self.compact else inf.grid_total)
 
     def set_solid_angle(self, normals, elem, omega0):
         """Exact back projection (Sec. II-C): weight every term by the share of
@@ -178,13 +188,16 @@ class BP:
                 raise ValueError("scales must be [F, ns]")
         if out is None:
             out = torch.empty(self.out_shape(F), dtype=torch.float32, device=signals.device)
-        elif not out.is_contiguous() or out.dtype != torch.float32 or out.numel() != int(
-                np.prod(self.out_shape(F))):
+        elif not out.is_contiguous() or out.dtype != torch.float32 or \
+                out.numel() != F * self._frame_numel:
             raise ValueError("out must be a contiguous float32 tensor of the output shape")
-        _lib.check(self._lib.pat_bp_reconstruct(
-            self._h, ctypes.c_void_p(signals.data_ptr()), code,
-            None if scales is None else ctypes.c_void_p(scales.data_ptr()), F,
-            ctypes.c_void_p(out.data_ptr()), _stream_ptr(stream)), "pat_bp_reconstruct")
+        # plain integers and no NumPy on this path: a small frame's kernels take
+        # less time than a careless call (pointers are converted by argtypes)
+        status = self._lib.pat_bp_reconstruct(
+            self._h, signals.data_ptr(), code, None if scales is None else scales.data_ptr(), F,
+            out.data_ptr(), _stream_ptr(stream))
+        if status:
+            _lib.check(status, "pat_bp_reconstruct")
         return out
 
     def preprocess(self, signals, scales=None, stream=None):

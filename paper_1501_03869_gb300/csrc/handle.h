@@ -52,6 +52,7 @@ struct pat_bp_s {
   // launch shapes chosen by the autotuner: [frames-per-group index][format]
   int tuned_S[6][3] = {};
   int tuned_budget_kb[6][3] = {};
+  int direct_fits[3][2] = {};         // unstaged launches per (format, weights): 1 fit, 2 do not, 0 unknown
   float* d_u = nullptr;               // table offsets (delays == 0)
   float* d_anchor = nullptr;          // per (tile, sensor) anchors (delays == 1)
   float4* d_pix = nullptr;            // per-pixel terms (delays == 1 or wgt)

@@ -732,8 +732,7 @@ cudaError_t launch_gather(const GatherConfig& c, int fmt, const StreamParams& p,
       df.b = static_cast<const unsigned char*>(d.b) + size_t(f) * d.n_sensors * d.n_t_pad * word;
       df.m = d.m + size_t(f) * d.n_sensors_pad;
       df.out = d.out + int64_t(f) * d.out_stride;
-      cudaError_t e = launch_gather_direct(c, fmt, df, c.n_sm, p.status,
-                                           f + 1 == d.n_frames ? p.host_status : nullptr, p.timeout_ns, st);
+      cudaError_t e = launch_gather_direct(c, fmt, df, c.n_sm, p.status, nullptr, p.timeout_ns, st);
       if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

@@ -77,8 +77,6 @@ struct StreamParams {
   int split;                // batched gather: 1 = a unit is one segment of a tile (their sums
                             // are added by a second kernel), 0 = all segments of a tile
   int* status;
-  int* host_status;         // host-mapped word the unstaged path's last kernel copies the
-                            // status into, or NULL
   unsigned* sched;          // [4] zero-initialised: unit ticket (64-bit) and CTAs finished
   uint64_t timeout_ns;
 };

@@ -806,6 +806,25 @@ static pat_status gather_locked(pat_bp_t h, int n_frames, float* out_dev, cudaSt
   int wst = 0;
   const GatherConfig c = pick_config(h, n_frames, h->pre_fmt, &wst);
   if (c.FB != h->pre_fb) return fail(PAT_ERR_INVALID, "frame grouping changed since preprocess");
+  if (c.direct) {
+    // one frame after the other, without the many-instance parameter block:
+    // frame f's integrand rows and multipliers are frame group f of the
+    // one-frame-per-group layout, the partial sums are reused
+    int& fits = h->direct_fits[h->pre_fmt][h->wgt];
+    if (!fits) fits = resident_ctas(c, h->pre_fmt, wst, h->n_sm) > 0 ? 1 : 2;
+    if (fits == 2) return fail(PAT_ERR_CUDA, "gather kernel does not fit on the device");
+    if (exported) *exported = host_status != nullptr;
+    InstDesc d = make_desc(h, out_dev, 1, 1, wst);
+    for (int f = 0; f < n_frames; ++f) {
+      cudaError_t e = launch_gather_direct(c, h->pre_fmt, d, c.n_sm, h->d_status,
+                                           f + 1 == n_frames ? host_status : nullptr, 2000000000ull, stream);
+      if (e != cudaSuccess) return cuda_fail(e, "gather launch");
+      d.b = static_cast<const unsigned char*>(d.b) + size_t(h->ns) * h->nt_pad * 4;  // 32-bit words in every format
+      d.m += h->ns_pad;
+      d.out += d.out_stride;
+    }
+    return PAT_OK;
+  }
   StreamParams sp;
   std::memset(&sp, 0, sizeof(sp));
   sp.inst[0] = make_desc(h, out_dev, n_frames, c.FB, wst);
@@ -818,8 +837,7 @@ static pat_status gather_locked(pat_bp_t h, int n_frames, float* out_dev, cudaSt
   sp.stages = c.stages;
   sp.Wst = wst;
   sp.status = h->d_status;
-  sp.host_status = c.direct ? host_status : nullptr;
-  if (exported) *exported = c.direct && host_status;
+  if (exported) *exported = false;
   sp.sched = h->d_sched;
   sp.timeout_ns = 2000000000ull;
   const int res = resident_ctas(c, h->pre_fmt, wst, h->n_sm);
