@@ -608,11 +608,14 @@ cudaError_t launch_window_w(int fmt, const DirectParams& dp, int n_sm, cudaStrea
 // The smallest slot (128, 192, 288 or 384 rows) that holds every window.
 template <int P, int SW, int DELAYS, int WGT>
 cudaError_t launch_window(int fmt, const DirectParams& dp, int n_sm, cudaStream_t st, bool reduce) {
-  if (dp.W <= 128) return launch_window_w<P, SW, 128, DELAYS, WGT>(fmt, dp, n_sm, st, reduce);
-  if (dp.W <= 192) return launch_window_w<P, SW, 192, DELAYS, WGT>(fmt, dp, n_sm, st, reduce);
+  if constexpr (DELAYS == 0 || P == 128) {
+    if (dp.W <= 128) return launch_window_w<P, SW, 128, DELAYS, WGT>(fmt, dp, n_sm, st, reduce);
+    if (dp.W <= 192) return launch_window_w<P, SW, 192, DELAYS, WGT>(fmt, dp, n_sm, st, reduce);
+  }
   if constexpr (DELAYS == 0 && WGT == 0)
     if (dp.W > 288) return launch_window_w<P, SW, kWindowMaxRows, 0, 0>(fmt, dp, n_sm, st, reduce);
-  return launch_window_w<P, SW, 288, DELAYS, WGT>(fmt, dp, n_sm, st, reduce);
+  if constexpr (DELAYS == 0) return launch_window_w<P, SW, 288, DELAYS, WGT>(fmt, dp, n_sm, st, reduce);
+  return cudaErrorInvalidValue;
 }
 
 template <int P, int SW>
@@ -671,11 +674,13 @@ cudaError_t launch_gather_direct(const GatherConfig& c, int fmt, const InstDesc&
   dp.n_seg = d.n_seg;
   dp.G = d.G;
   dp.W = d.W;
-  // the windowed kernel when every window fits a slot.  Computed delays and
-  // weights hold more registers (6 CTAs per SM): with slots of 384 rows they
-  // lose to the kernel above (paper-shaped frame at constant speed 30.0 us
-  // against 28.4; stored table with 256-pixel tiles 26.1 -> 22.9)
-  const int most = c.delays || dp.wanchor ? 288 : kWindowMaxRows;
+  // The windowed kernel when every window fits a slot.  Weights and computed
+  // delays hold more registers (6 CTAs per SM), and with computed delays the
+  // kernel above reads little besides the integrand: weights up to 288 rows
+  // (272 rows: 32.0 -> 30.7 us), computed delays up to 192 rows of 128-pixel
+  // tiles (120 rows: 549 -> 422 us; 360 rows 28.4 against 30.0, 256-pixel tiles
+  // 25.1 against 26.3).
+  const int most = c.delays ? (c.P == 128 ? 192 : 0) : (dp.wanchor ? 288 : kWindowMaxRows);
   const bool window = !c.no_window && dp.W >= 0 && dp.W <= most && dp.G <= 64;
   if (window && c.P == 128 && c.SW == 4) return launch_window_mode<128, 4>(c.delays != 0, fmt, dp, n_sm, st, reduce);
   if (window && c.P == 256 && c.SW == 2) return launch_window_mode<256, 2>(c.delays != 0, fmt, dp, n_sm, st, reduce);

@@ -450,6 +450,30 @@ __global__ void __launch_bounds__(RowsShape<P, FB, FMT>::THREADS, RowsShape<P, F
     uint32_t quad[NQ];  // byte offsets of the lane's quads in a row
 #pragma unroll
     for (int k = 0; k < NQ; ++k) quad[k] = uint32_t(lq) * 16u + (NQ == 2 ? (uint32_t(k) ^ (uint32_t(g) & 1u)) * (ROW / 2u) : 0u);
+    // Computed offsets and weights are the same for the LPP lanes of a pixel: a
+    // lane evaluates them for pixels i * 32 + lane of its warp and the lanes of
+    // a pixel fetch them by shuffles where that saves evaluations (64 FP32
+    // constant-speed frames, 256-pixel tiles: 437 -> 380 us; not for 16-frame
+    // rows with computed delays, whose two pixels per lane save too little:
+    // 181 us against 191).
+    constexpr bool SHARE = A > (NPX + 31) / 32 && (FB != 16 || MODE == 2);
+    constexpr int NV = SHARE ? (NPX + 31) / 32 : A;
+    auto spread = [&](const float (&mine)[NV], float (&of)[A]) {
+#pragma unroll
+      for (int a = 0; a < A; ++a) {
+        if constexpr (!SHARE) {
+          of[a] = mine[a];
+          continue;
+        }
+        const int l = pixel(a) - warp * NPX;
+        float v = __shfl_sync(0xffffffffu, mine[0], l & 31);
+        if constexpr (SHARE && NV > 1) {
+          const float v1 = __shfl_sync(0xffffffffu, mine[1], l & 31);
+          v = l < 32 ? v : v1;
+        }
+        of[a] = v;
+      }
+    };
     const uint32_t u_lane = uint32_t(warp * NPX + g * V) * 4u;
     int inst = 0;
     int st = 0;             // slot in use and the parity of its next completion
@@ -469,10 +493,10 @@ __global__ void __launch_bounds__(RowsShape<P, FB, FMT>::THREADS, RowsShape<P, F
       if (u < 0) break;
       const RowsUnit q = decode_rows(p, u, inst);
       const InstDesc& d = p.inst[q.inst];
-      float4 pq[A];  // constant speed or weights: the lane's pixels relative to the tile anchor
+      float4 pq[NV];  // constant speed or weights: pixels relative to the tile anchor
       if constexpr (DELAYS != 0 || WGT != 0) {
 #pragma unroll
-        for (int a = 0; a < A; ++a) pq[a] = __ldcg(d.pix + int64_t(q.tile) * P + pixel(a));
+        for (int i = 0; i < NV; ++i) pq[i] = __ldcg(d.pix + int64_t(q.tile) * P + (SHARE ? warp * NPX + (i * 32 + lane) % NPX : pixel(i)));
       }
       bool first = true;
       for (int seg = q.seg0; seg < q.seg1 && ok; ++seg) {
@@ -527,7 +551,9 @@ __global__ void __launch_bounds__(RowsShape<P, FB, FMT>::THREADS, RowsShape<P, F
             const float lim = __uint_as_float(h.rec.y);
             if constexpr (DELAYS != 0) {
               const float4* sa = reinterpret_cast<const float4*>(ring + hdr.x) + 2 * sl;
-              constant_offsets<A>(h.uu, pq, sa[0], sa[1]);
+              float mine[NV];
+              constant_offsets<NV>(mine, pq, sa[0], sa[1]);
+              spread(mine, h.uu);
             }
             // floor and phase from the FP32 bits: u + 2^23 rounded toward
             // zero is 2^23 + floor(u), whose low bits are floor(u)
@@ -546,19 +572,19 @@ __global__ void __launch_bounds__(RowsShape<P, FB, FMT>::THREADS, RowsShape<P, F
                 row[a] += swap[a] * ROW;
               }
             }
-            float4 E, Nn;
+            float ww[A];
             if constexpr (WGT != 0) {
               const float4* wa = reinterpret_cast<const float4*>(ring + hdr.x + L.wa) + 2 * sl;
-              E = wa[0];
-              Nn = wa[1];
+              const float4 E = wa[0], Nn = wa[1];
+              float mine[NV];
+#pragma unroll
+              for (int i = 0; i < NV; ++i) mine[i] = solid_angle_weight(pq[i], E, Nn);
+              spread(mine, ww);
             }
 #pragma unroll
             for (int a = 0; a < A; ++a) {
               f32x2 wp = 0ull;
-              if constexpr (WGT != 0) {
-                const float w = solid_angle_weight(pq[a], E, Nn);
-                wp = pack2(w, w);
-              }
+              if constexpr (WGT != 0) wp = pack2(ww[a], ww[a]);
               // swapped rows: x is b_{k+1} and y is b_k, so y - x is the exact
               // negative of the slope and the phase changes sign with it
               const float sp = PAR ? __uint_as_float(__float_as_uint(ph[a]) ^ (swap[a] << 31)) : ph[a];

@@ -383,6 +383,9 @@ int frames_per_unit(pat_bp_t h, int n_frames) {
   // frames of 6 092 pixels x 64 sensors: 41 us in rows of 32 (96 units), 34 of
   // 16, 32 of 8, 43 of 4; 5 000 pixels x 256 sensors: 157, 121, 139, 125.
   int FB = frames_per_group(n_frames);
+  // computed delays and weights together outweigh what 16-frame rows save (12
+  // FP16 frames: 181 us in rows of 16, 174 of 8)
+  if (h->delays && h->wgt && h->P == 128 && FB == 16) FB = 8;
   while (FB > 4) {
     const int64_t units = int64_t((n_frames + FB - 1) / FB) * h->n_tiles * h->n_seg;
     if (units >= int64_t(FB == 8 ? 1 : 4) * h->n_sm) break;
