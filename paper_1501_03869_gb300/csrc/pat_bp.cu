@@ -423,7 +423,11 @@ static pat_status grow_zeroed(void** p, size_t* cap, size_t need, const char* wh
 pat_status ensure_buffers_fb(pat_bp_t h, int n_frames, int FB) {
   const size_t n_fg = size_t((n_frames + FB - 1) / FB);
   pat_status st;
-  const size_t b_need = (n_fg * h->ns * h->nt_pad + kTailRows) * FB * 4;
+  // The slack rows and the counters do not depend on FB from 4 frames on: a
+  // reservation made for long rows also holds a launch that takes shorter ones
+  // (frames_per_unit), which may be under capture.
+  const int tail = FB < 4 ? FB : 32, cnt_fb = std::min(FB, 4);
+  const size_t b_need = (n_fg * h->ns * h->nt_pad * FB + size_t(kTailRows) * tail) * 4;
   if ((st = grow_zeroed(&h->d_b, &h->b_cap, b_need, "integrand buffer")) != PAT_OK) return st;
   const size_t m_need = n_fg * h->ns_pad * FB * sizeof(float);
   if ((st = grow_zeroed(reinterpret_cast<void**>(&h->d_m), &h->m_cap, m_need, "multipliers")) != PAT_OK)
@@ -435,7 +439,7 @@ pat_status ensure_buffers_fb(pat_bp_t h, int n_frames, int FB) {
     if ((st = grow_zeroed(reinterpret_cast<void**>(&h->d_part), &h->part_cap, part_need,
                           "segment partials")) != PAT_OK)
       return st;
-    const size_t cnt_need = n_fg * h->n_tiles * sizeof(int);
+    const size_t cnt_need = size_t((n_frames + cnt_fb - 1) / cnt_fb) * h->n_tiles * sizeof(int);
     if ((st = grow_zeroed(reinterpret_cast<void**>(&h->d_counter), &h->counter_cap, cnt_need,
                           "segment counters")) != PAT_OK)
       return st;

@@ -107,3 +107,24 @@ def test_non_finite_frame_stays_alone():
         sig[3, 10, 40:60] = float("inf")
         sig[3, 11, 100] = float("nan")
         _check(bp, sig, None, (2, 3, 4, 31))
+
+
+@pytest.mark.parametrize("reserved,frames", [(64, 64), (32, 32), (16, 16), (40, 32), (64, 17), (24, 8)])
+def test_reserved_handle_allocates_nothing_for_shorter_rows(reserved, frames):
+    """A small launch takes shorter rows than its frame count allows; what
+    reserve() set aside for the longest ones holds it, so that its first call
+    can already be under capture."""
+    with _handle((72, 80), 64, 301, 128, "table") as bp, _handle((72, 80), 64, 301, 128, "table") as ref:
+        sig, _ = _signals(frames, 64, 301, "f32")
+        want = ref.reconstruct(sig)
+        bp.reserve(reserved)
+        out = torch.empty_like(want)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            bp.reconstruct(sig, out=out)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out.view(torch.int32), want.view(torch.int32))
+        bp.sync()
+        ref.sync()
