@@ -469,11 +469,18 @@ bool gpu_eikonal_slot_times(GpuEikonal* e, const double* sensors, int nb, double
   // Rounds accept lowerings up to tau = (round + 1) * dtau (a bucketed
   // Dijkstra order): a node takes a value only once the values upwind of it
   // are final or nearly so, instead of passing provisional values far ahead
-  // of the front.  dtau is a quarter block edge of the mean medium (8 x 8 x 4
-  // blocks: two node spacings; 16 x 16: four), or 1/1024 of the time span
-  // when that is coarser.
+  // of the front.  dtau is a part of the block edge of the mean medium, or
+  // 1/1024 of the time span when that is coarser: a quarter for 8 x 8 x 4
+  // blocks (two node spacings, the best of those tried), half for 16 x 16
+  // (eight).  A 2-D sweep does little work beside its round's list, two
+  // launches and wait, so fewer rounds win until values are passed on too
+  // early.  Quarter / three eighths / half / five eighths, whole call:
+  // 128 x 128, 64 sources 3.47 / 3.02 / 2.82 / 2.65 ms; 200 x 200, 100
+  // sources 10.8 / 9.2 / 8.3 / 8.0; 384 x 384, 32 sources 13.9 / 12.2 / 11.4
+  // / 11.3; the table of 256 x 256 with 512 sensors builds in 49 ms instead
+  // of 63.
   const double t_end = std::min(stop_after, double(g.n[0] + g.n[1] + g.n[2]) * e->hf_max);
-  const double dtau = std::max(0.25 * e->B[0] * e->hf_mean, t_end / 1024.0);
+  const double dtau = std::max((g.ndim == 2 ? 0.5 : 0.25) * e->B[0] * e->hf_mean, t_end / 1024.0);
   for (int d = 0; d < 3; ++d) {
     p.n[d] = g.n[d];
     p.bn[d] = e->bn[d];
