@@ -1,0 +1,58 @@
+"""One frame through the windowed gather and through the kernel that reads the
+integrand from L2 (PAT_FLAG_NO_WINDOW): the same bits for every kind of delay
+and weight, tile size and format, with windows on both sides of each slot size
+(128, 192, 288 and 384 rows, and longer ones that take the other kernel), one
+ragged segment of sensors (the gather writes the image) and two."""
+import numpy as np
+import pytest
+
+from paper_1501_03869_gb300 import BP, _lib, synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
+def _handle(mode, tile, ns, nt, extra):
+    rng = np.random.default_rng(5)
+    shape, dx = (64, 70), 0.2e-3
+    speed = (1500.0 + 900.0 * synth.smooth_field(shape, 4.0, rng)).astype(np.float32)
+    hi = (np.array(shape[::-1], dtype=float) - 1) * dx
+    sensors = np.zeros((ns, 3))
+    sensors[:, 0] = np.where(np.arange(ns) % 2, hi[0], 0.0)
+    sensors[:, 1] = (np.floor(rng.uniform(0.0, 1.0, ns) * (shape[0] - 2)) + 0.37) * dx  # off the nodes
+    dt = 1.2 * float(np.linalg.norm(hi)) / 1500.0 / nt
+    flags = extra | (_lib.PAT_FLAG_TILE_256 if tile == 256 else _lib.PAT_FLAG_TILE_128)
+    if mode.startswith("constant"):
+        bp = BP.constant(1560.0, shape, dx, np.zeros(3), sensors, dt, nt, flags=flags)
+    else:
+        bp = BP(speed, dx, np.zeros(3), sensors, dt, nt, flags=flags)
+    if mode.endswith("solid"):
+        normals = np.zeros((ns, 3))
+        normals[:, 0] = np.where(np.arange(ns) % 2, -1.0, 1.0)
+        bp.set_solid_angle(normals, np.full(ns, dx), 2 * np.pi)
+    return bp
+
+
+@pytest.mark.parametrize("nt", [600, 1000, 1199, 1600, 2000, 2400])
+@pytest.mark.parametrize("tile", [128, 256])
+@pytest.mark.parametrize("mode", ["table", "constant", "table_solid", "constant_solid"])
+def test_windowed_equals_unwindowed(mode, tile, nt):
+    for ns in (37, 70):
+        g = torch.Generator("cuda").manual_seed(nt + ns)
+        x = torch.randn(1, ns, nt, generator=g, device="cuda")
+        sc = x.abs().amax(dim=2).contiguous()
+        with _handle(mode, tile, ns, nt, 0) as a, _handle(mode, tile, ns, nt, _lib.PAT_FLAG_NO_WINDOW) as b:
+            for dtype in (torch.float32, torch.bfloat16, torch.float16):
+                s = None if dtype == torch.float32 else sc
+                sig = x if s is None else (x / sc[..., None]).to(dtype).contiguous()
+                ia, ib = a.reconstruct(sig, scales=s), b.reconstruct(sig, scales=s)
+                assert torch.isfinite(ia).all() and bool((ia != 0).any())
+                assert torch.equal(ia.view(torch.int32), ib.view(torch.int32)), (ns, dtype, a.info["window"])
+            a.sync()
+            b.sync()
