@@ -78,12 +78,13 @@ typedef void* pat_stream_t; /* a cudaStream_t; NULL = legacy default stream */
                                          pipeline) gather too; by default one
                                          frame takes the unstaged kernel, which
                                          gives the same bits                     */
-#define PAT_FLAG_NO_WINDOW 0x1000u /* unstaged single frames of a stored table
-                                      gather the integrand from L2 instead of
-                                      from shared-memory windows (the default
-                                      whenever every window of the table has at
-                                      most 288 samples); same bits, for
-                                      comparisons                               */
+#define PAT_FLAG_NO_WINDOW 0x1000u /* unstaged single frames gather the
+                                      integrand from L2 instead of from
+                                      shared-memory windows (the default
+                                      whenever every window has at most 384
+                                      samples; 288 with solid-angle weights;
+                                      constant speed: 192, and 128 pixels per
+                                      tile); same bits, for comparisons         */
 
 /* Read-only facts about a handle (pat_bp_info). */
 typedef struct {
@@ -291,10 +292,11 @@ pat_status pat_table_host(const float* speed_host, const pat_grid* grid, const d
  * Many instances in persistent launches (uneven grids, sensor counts, sample
  * counts and frame counts).  A plan fixes the handles and their frame counts
  * and groups the instances by frames per unit FB (the largest power of two up
- * to 8 not above an instance's frame count: FB frames share each pass over a
- * table tile).  Each execution runs one preprocessing launch per group, then
- * one persistent gather launch per group (the first programmatically
- * dependent on the preprocessing), optionally replayed as a CUDA graph.  The
+ * to 8 not above an instance's frame count; 16 or 32 above 16 frames where that
+ * pads no further: FB frames share each pass over a table tile).  Each
+ * execution runs one preprocessing launch per group, then one persistent gather
+ * launch per group (the first programmatically dependent on the preprocessing;
+ * from 4 frames on followed by the segment sums), optionally replayed as a CUDA graph.  The
  * summation order of every instance is its handle's own, so each image is
  * bit-identical to that handle's pat_bp_reconstruct of the same frames,
  * whatever else is in the plan or however the launches are shaped.
