@@ -151,7 +151,7 @@ def kernel_source_hash():
     """Hash of the sources of the single-frame gather (the kernel the roofline
     line is about); a committed traffic record is used only while it matches."""
     h = hashlib.sha256()
-    for fn in ("gather_direct.cu", "gather.cuh", "kernels.cuh", "device.cuh"):
+    for fn in ("gather_direct.cu", "packed.cuh", "gather.cuh", "kernels.cuh", "device.cuh"):
         with open(os.path.join(ROOT, "paper_1501_03869_gb300", "csrc", fn), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -159,12 +159,12 @@ def kernel_source_hash():
 
 def single_frame_kernels(info):
     """Names of the two kernels one FP32 frame of a stored table takes: the
-    windowed gather when every window fits its largest slot (288 rows)."""
+    windowed gather when every window fits its largest slot (384 rows)."""
     P = info["tile_pix"]
     sw = 4 if P == 128 else 2
     W = info["window"]
-    if W <= 288:
-        wb = 128 if W <= 128 else (192 if W <= 192 else 288)
+    if W <= 384:
+        wb = next(b for b in (128, 192, 288, 384) if W <= b)
         return f"gather_window_kernel<{P},{sw},f32,{wb}> + direct_reduce_kernel<{P},1>"
     return f"gather_direct_kernel<{P},{sw},f32,table> + direct_reduce_kernel<{P},{sw}>"
 
@@ -636,7 +636,7 @@ def constant_form(args, w, flush, stream, checks):
 
 
 def batched_roofline(w, tile_flags, F, FB, shared_read_bytes, gather_ms, sm_mhz, n_sm, l2_smem_gbs):
-    """Roofline of the staged gather on F frames: the larger of the
+    """Roofline of the batched gather on F frames: the larger of the
     shared-memory time (gather reads plus the bulk copies' writes, 128 B per
     clock per SM) and the L2 -> shared stream time (window and table-block
     copies against the measured bulk-copy bandwidth), against the measured
@@ -1066,7 +1066,7 @@ def main():
                 return e0, e1, e2
             rg = time_steps(gstep, n_rep, 2, stream, flush)
             g_ms = statistics.mean(b.elapsed_time(c) for a, b, c in rg)
-            FB = min(8, 1 << (F.bit_length() - 1))
+            FB = min(32, 1 << (F.bit_length() - 1))  # 64 frames of this geometry: rows of 32
             forms[name] = {"frames": F, "ms_per_batch": ms, "frames_per_s": F / (ms / 1e3),
                            "value": F * updates / (ms / 1e3) / 1e9, "unit": UNIT, "tile_pix": 256,
                            "gather_ms": g_ms,

@@ -19,7 +19,7 @@
 // Measured, whole calls (preprocessing and reduction included): 64 FP32 frames
 // of 512 sensors x 21 323 pixels 489 -> 346 us; 8 BF16 frames of 640 sensors x
 // 1.04 M voxels 3.17 -> 2.12 ms; 64 BF16 frames of 64 x 6 092 54 -> 33 us; 12
-// FP16 frames with solid-angle weights 166 -> 137 us.
+// FP16 frames with solid-angle weights 166 -> 136 us.
 //
 // Work: one unit is (frame group, tile) with all segments of G sensors when
 // there are many units, else (frame group, tile, segment), whose sums
