@@ -39,6 +39,7 @@
 
 #include "gather.cuh"
 #include "packed.cuh"
+#include "rows_layout.h"
 
 namespace patbp {
 
@@ -59,41 +60,6 @@ struct RowsShape {
   // resident CTAs per SM the registers must allow: 11 to 18 warps
   static constexpr int MIN_CTAS = FB >= 16 ? 1 : 3;
   static_assert(A % V == 0 && NPX * NW == P, "pixels of a lane");
-};
-
-// Shared memory: header, then a ring of StreamParams::ring bytes that is filled
-// with groups of S consecutive sensors (kSlots of them at most), then 2 zero
-// rows that out-of-record pixels read, then the running sums of whole-tile
-// units.  A group takes the bytes it needs: windows differ threefold between
-// tiles and sensors, and fixed stages sized for the longest sum left two or
-// three stages in flight.
-//   u    [se][P] float    table rows, or [se][8] float anchors (constant speed)
-//   wa   [se][8] float    solid-angle weight anchors (mode bit 1 only)
-//   m    [se][FB] float   multipliers w_s * sigma
-//   rec  [se] uint2       window address and row limit of each sensor
-//   win  [rows][FB]       the windows back to back (128-byte aligned)
-constexpr int kSlots = 8;
-constexpr int kRowsMaxS = 16;  // sensors of a group
-constexpr int kSegs = 10;      // segments alive: one per slot, one being planned, one spare
-struct RowsSegment {           // what the copiers need of a (unit, segment)
-  uint2 sensor[64];            // (window base | length << 16, rows of the segment before it)
-  uint64_t u, wa, b, m;        // addresses of the segment's first sensor
-  uint64_t stride;             // bytes from one sensor's integrand rows to the next's
-  uint64_t pad;
-};
-constexpr int kRowsBars = 512;
-constexpr int kRowsHeader = (kRowsBars + 2 * 64 * 4 + kSegs * int(sizeof(RowsSegment)) + 127) / 128 * 128;
-struct RowsGroup {
-  uint32_t wa, m, rec, win;
-  __host__ __device__ RowsGroup(int se, int P, int FB, int mode) {
-    wa = (mode & 1) ? uint32_t(se) * 32u : uint32_t(se) * uint32_t(P) * 4u;
-    m = wa + ((mode & 2) ? uint32_t(se) * 32u : 0u);
-    rec = m + uint32_t(se) * uint32_t(FB) * 4u;
-    win = (rec + uint32_t(se) * 8u + 127u) & ~127u;
-  }
-  __host__ __device__ uint32_t bytes(int rows, int FB) const {
-    return (win + uint32_t(rows) * uint32_t(FB) * 4u + 127u) & ~127u;
-  }
 };
 
 struct RowsUnit {
@@ -135,8 +101,9 @@ __global__ void __launch_bounds__(RowsShape<P, FB, FMT>::THREADS, RowsShape<P, F
   uint4* slot_hdr = reinterpret_cast<uint4*>(unit_ring + kRing);  // [kSlots] (ring offset, sensors, first
                                                                   // sensor | segment << 16, rows)
   volatile int* abort_flag = reinterpret_cast<volatile int*>(slot_hdr + kSlots);
-  uint32_t* meta = reinterpret_cast<uint32_t*>(smem + kRowsBars);  // [2][64] packed bases
-  RowsSegment* segs = reinterpret_cast<RowsSegment*>(meta + 2 * 64);
+  uint32_t* meta = reinterpret_cast<uint32_t*>(smem + kRowsMeta);  // [2][64] packed bases
+  RowsRecord* recs = reinterpret_cast<RowsRecord*>(smem + kRowsRecs);  // [kSlots][kRowsMaxS]
+  RowsSegment* segs = reinterpret_cast<RowsSegment*>(smem + kRowsSegs);
   unsigned char* ring = smem + kRowsHeader;
   float* total = reinterpret_cast<float*>(ring + p.ring + 2 * ROW);  // [P][FB], whole-tile units
   const uint32_t ring_s = smem_addr(ring);
@@ -187,16 +154,16 @@ __global__ void __launch_bounds__(RowsShape<P, FB, FMT>::THREADS, RowsShape<P, F
       uint64_t src = 0;
       uint32_t dst = 0, bytes = 0;
       if (lane < se) {
-        const uint2 x = sg.sensor[i0 + lane];
+        const RowsSensor x = sg.sensor[i0 + lane];
         const bool bad = hdr.w == 0xffffffffu;  // no room for the windows (a configuration error)
-        const uint32_t w = bad ? uint32_t(p.ring) : hdr.x + L.win + (x.y - sg.sensor[i0].y) * ROW;
+        const uint32_t w = bad ? uint32_t(p.ring) : hdr.x + L.win + (x.before - sg.sensor[i0].before) * ROW;
         // row r of the sensor's window is at rec.x + ROW * (2^23's bits + r);
         // the zero rows follow the ring
-        reinterpret_cast<uint2*>(ring + hdr.x + L.rec)[lane] =
-            make_uint2(ring_s + w - kMagic * ROW, __float_as_uint(float((uint32_t(p.ring) - w) / ROW)));
-        src = sg.b + uint64_t(i0 + lane) * sg.stride + uint64_t((x.x & 0xffffu) * ROW);
+        recs[slot * kRowsMaxS + lane] =
+            RowsRecord{ring_s + w - kMagic * ROW, __float_as_uint(float((uint32_t(p.ring) - w) / ROW))};
+        src = sg.b + uint64_t(i0 + lane) * sg.stride + uint64_t((x.base_len & 0xffffu) * ROW);
         dst = ring_s + w;
-        bytes = bad ? 0u : (x.x >> 16) * ROW;
+        bytes = bad ? 0u : (x.base_len >> 16) * ROW;
       } else if (lane == 16) {
         src = sg.u + uint64_t(i0) * (DELAYS ? 32u : P * 4u);
         dst = ring_s + hdr.x;
@@ -305,7 +272,7 @@ __global__ void __launch_bounds__(RowsShape<P, FB, FMT>::THREADS, RowsShape<P, F
       if (lane == 0) {
         slot_hdr[next] = make_uint4(at, uint32_t(se), uint32_t(i0) | uint32_t(sg) << 16, bad ? 0xffffffffu : rows);
         if (bad) atomicOr(p.status, kStatusBadConfig);
-        mbar_arrive_expect_tx(&full[next], L.rec + rows * ROW);
+        mbar_arrive_expect_tx(&full[next], L.copied(int(rows), FB));
         mbar_arrive(&plan_bar[next]);
       }
       ++n_fly;
@@ -371,8 +338,8 @@ __global__ void __launch_bounds__(RowsShape<P, FB, FMT>::THREADS, RowsShape<P, F
         }
         a1 += __shfl_sync(0xffffffffu, a0, 31);
         RowsSegment& sg = segs[sgi];
-        sg.sensor[lane] = make_uint2(w0, a0 - (w0 >> 16));
-        sg.sensor[lane + 32] = make_uint2(w1, a1 - (w1 >> 16));
+        sg.sensor[lane] = RowsSensor{w0, a0 - (w0 >> 16)};
+        sg.sensor[lane + 32] = RowsSensor{w1, a1 - (w1 >> 16)};
         if (lane == 0) {
           sg.u = DELAYS ? reinterpret_cast<uint64_t>(d.anchor + (int64_t(q.tile) * d.n_sensors_pad + s_lo) * 8)
                         : reinterpret_cast<uint64_t>(d.u + (int64_t(q.tile) * d.n_sensors + s_lo) * P);
@@ -518,14 +485,14 @@ __global__ void __launch_bounds__(RowsShape<P, FB, FMT>::THREADS, RowsShape<P, F
           const int se = int(hdr.y);
           const RowsGroup L(se, P, FB, MODE);
           const uint32_t sb = ring_s + hdr.x;
-          const uint32_t m_at = sb + L.m;
+          const uint32_t m_at = sb + L.m, rec_at = smem_addr(recs + st * kRowsMaxS);
           struct Head {  // what a sensor needs before its rows
             uint2 rec;
             f32x2 m[2 * NQ];
             float uu[A];
           };
           auto load_head = [&](Head& h, int sl) {
-            h.rec = lds_u2(sb + L.rec + uint32_t(sl) * 8u);
+            h.rec = lds_u2(rec_at + uint32_t(sl) * 8u);
 #pragma unroll
             for (int k = 0; k < NQ; ++k) lds_2x64(m_at + uint32_t(sl) * ROW + quad[k], h.m[2 * k], h.m[2 * k + 1]);
             if constexpr (DELAYS == 0) {

@@ -1,0 +1,24 @@
+"""The shared-memory layout of the batched gather, on CPU
+(tests/native/rows_layout.cpp): bulk copies fill a group's place in the ring
+without a byte left for ordinary stores, which the memory model would not order
+against a later group's copies."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1501_03869_gb300", "csrc")
+
+
+def test_ring_holds_bulk_copied_bytes_only(tmp_path):
+    gxx = shutil.which("g++")
+    if not gxx:
+        pytest.skip("g++ not found")
+    exe = str(tmp_path / "rows_layout")
+    src = os.path.join(ROOT, "tests", "native", "rows_layout.cpp")
+    r = subprocess.run([gxx, "-std=c++17", "-Wall", f"-I{CSRC}", src, "-o", exe], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-3000:]
+    r = subprocess.run([exe], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout[-3000:]
