@@ -33,6 +33,7 @@
 
 #include "device.cuh"
 #include "kernels.cuh"
+#include "smem_grant.h"
 
 namespace patbp {
 
@@ -662,16 +663,23 @@ __global__ void __launch_bounds__(32 * ((P / 128) * SW + 3), (MODE & 1) ? (FB ==
 }
 
 // ------------------------------------------------------- launch templates --
+// Lets `kern` take `smem` bytes of dynamic shared memory on the current device.
+template <class K>
+static cudaError_t grant_smem(SmemGrant& grant, K* kern, size_t smem) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  return grant.ensure(dev, smem, [&](size_t bytes) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
+  });
+}
+
 template <int P, int FB, int FMT, int SW, int MODE>
 static cudaError_t gather_t(const StreamParams& p, size_t smem, int grid, cudaStream_t st,
                             int* resident, int n_sm) {
   auto kern = gather_kernel<P, FB, FMT, SW, MODE>;
-  static size_t smem_set = 0;  // largest dynamic smem granted so far (per instantiation)
-  if (smem > smem_set) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e != cudaSuccess) return e;
-    smem_set = smem;
-  }
+  static SmemGrant grant;
+  if (cudaError_t e = grant_smem(grant, kern, smem); e != cudaSuccess) return e;
   const int threads = 32 * ((P / 128) * SW + 3);
   if (resident) {
     int per_sm = 0;

@@ -733,12 +733,8 @@ static cudaError_t rows_t(const StreamParams& p, size_t smem, int grid, cudaStre
                           int n_sm) {
   using SH = RowsShape<P, FB, FMT>;
   auto kern = gather_rows_kernel<P, FB, FMT, SW, MODE>;
-  static size_t smem_set = 0;  // largest dynamic smem granted so far (per instantiation)
-  if (smem > smem_set) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e != cudaSuccess) return e;
-    smem_set = smem;
-  }
+  static SmemGrant grant;
+  if (cudaError_t e = grant_smem(grant, kern, smem); e != cudaSuccess) return e;
   if (resident) {
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, SH::THREADS, smem);
