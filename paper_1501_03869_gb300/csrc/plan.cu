@@ -58,6 +58,7 @@ struct pat_plan_s {
   unsigned flags = 0;
   int device = 0, n_sm = 0, P = 128, SW = 4;
   int fb_uniform = 0;  // 0: each instance's own frames per unit; else this for all
+  std::vector<int> fbs;  // frames per unit of every instance
   // launch shape shared by the classes
   int S = 16, budget_kb = 55;
   std::vector<PlanClass> cls;
@@ -85,13 +86,61 @@ int instance_fb(pat_plan_t pl, int i) {
   return F > 16 ? frames_per_group(F) : std::min(8, frames_per_group(F));
 }
 
+// Launch configuration of a class before its shape: mode and unit kind.
+GatherConfig class_config(pat_plan_t pl, const std::vector<int>& idx, int FB) {
+  GatherConfig c;
+  c.P = pl->P;
+  c.SW = pl->SW;
+  c.delays = pl->hs[0]->delays;
+  c.wgt = pl->hs[0]->wgt;
+  c.n_sm = pl->n_sm;
+  c.FB = FB;
+  int64_t tiles = 0;
+  int n_seg = 1;
+  for (int i : idx) {
+    tiles += int64_t((pl->frames[i] + FB - 1) / FB) * pl->hs[i]->n_tiles;
+    n_seg = std::max(n_seg, pl->hs[i]->n_seg);
+  }
+  set_units(c, tiles, n_seg);
+  return c;
+}
+
+// Longest window-row sum over the S-sensor groups of a class.
+int class_window(pat_plan_t pl, const std::vector<int>& idx, int S) {
+  int w = 8;
+  for (int i : idx) w = std::max(w, stage_window(pl->hs[i], S));
+  return w;
+}
+
+// Frames per unit of every instance.  Rows of 32 or 16 frames whose longest
+// window does not fit a CTA (32 frames: 1 752 rows) are halved down to 8, which
+// hold windows of almost 7 000.
+std::vector<int> choose_frames_per_unit(pat_plan_t pl) {
+  std::vector<int> fbs;
+  for (size_t i = 0; i < pl->hs.size(); ++i) fbs.push_back(instance_fb(pl, int(i)));
+  if (pl->fb_uniform) return fbs;
+  for (int FB = 32; FB > 8; FB /= 2) {
+    std::vector<int> idx;
+    for (size_t i = 0; i < fbs.size(); ++i)
+      if (fbs[i] == FB) idx.push_back(int(i));
+    if (idx.empty()) continue;
+    GatherConfig c = class_config(pl, idx, FB);
+    c.S = 1;
+    for (int i : idx) {
+      const int w = stage_window(pl->hs[i], 1);
+      int wst = w;
+      if (!fit_stages(c, w, w, size_t(pl->hs[0]->max_smem), &wst)) fbs[i] = FB / 2;
+    }
+  }
+  return fbs;
+}
+
 // Classes and launch shapes for S sensors per stage under a shared-memory
 // budget of budget_kb per CTA (0, 0: every class's own default shape).
 pat_status plan_shape(pat_plan_t pl, int S, int budget_kb) {
   pl->S = S;
   pl->budget_kb = budget_kb;
-  std::vector<int> fbs;
-  for (size_t i = 0; i < pl->hs.size(); ++i) fbs.push_back(instance_fb(pl, int(i)));
+  const std::vector<int>& fbs = pl->fbs;
   std::vector<int> order(fbs);
   std::sort(order.begin(), order.end(), std::greater<int>());
   order.erase(std::unique(order.begin(), order.end()), order.end());
@@ -114,39 +163,21 @@ pat_status plan_shape(pat_plan_t pl, int S, int budget_kb) {
     if (k.FB >= 4) Sk = std::min(Sk, 16);
     // one shape per class: the longest single window and the longest
     // S-sensor window sum of its instances bound the stages' row budget
-    int wmin = 8, wfull = 8;
-    for (int i : k.idx) {
-      wmin = std::max(wmin, stage_window(pl->hs[i], 1));
-      wfull = std::max(wfull, stage_window(pl->hs[i], Sk));
-    }
-    GatherConfig c;
-    c.P = pl->P;
-    c.SW = pl->SW;
-    c.delays = pl->hs[0]->delays;
-    c.wgt = pl->hs[0]->wgt;
-    c.n_sm = pl->n_sm;
-    c.FB = k.FB;
+    const int wmin = class_window(pl, k.idx, 1);
+    int wfull = class_window(pl, k.idx, Sk);
+    GatherConfig c = class_config(pl, k.idx, k.FB);
     c.S = Sk;
-    int64_t tiles = 0;
-    int n_seg = 1;
-    for (int i : k.idx) {
-      tiles += int64_t((pl->frames[i] + k.FB - 1) / k.FB) * pl->hs[i]->n_tiles;
-      n_seg = std::max(n_seg, pl->hs[i]->n_seg);
-    }
-    set_units(c, tiles, n_seg);
     int wst = wfull;
     bool fits = fit_stages(c, wmin, wfull, budget, &wst);
     if (k.FB >= 4)  // smaller groups of sensors where the longest sums do not fit
       while (!fits && c.S > 1) {
         c.S /= 2;
-        wfull = 8;
-        for (int i : k.idx) wfull = std::max(wfull, stage_window(pl->hs[i], c.S));
+        wfull = class_window(pl, k.idx, c.S);
         fits = fit_stages(c, wmin, wfull, budget, &wst);
       }
     if (!fits && S == 0 && budget < limit) {  // a default shape too small for long windows: the whole SM
       c.S = 4;
-      wfull = 8;
-      for (int i : k.idx) wfull = std::max(wfull, stage_window(pl->hs[i], c.S));
+      wfull = class_window(pl, k.idx, c.S);
       fits = fit_stages(c, wmin, wfull, limit, &wst);
     }
     if (!fits)
@@ -489,6 +520,7 @@ static pat_status plan_new(const pat_bp_t* handles, const int* n_frames, int n, 
   pl->P = handles[0]->P;
   pl->SW = handles[0]->SW;
   pl->fb_uniform = fb_uniform;
+  pl->fbs = choose_frames_per_unit(pl.get());
   PAT_CUDA(cudaSetDevice(pl->device));
   if (own_words) {
     if (cudaMalloc(&pl->d_status, sizeof(int)) != cudaSuccess ||

@@ -1,0 +1,82 @@
+"""Plans and handles whose batches take rows of 8 to 32 frames.  Every image has
+the bits of the same frames through the handle's own reconstruct() (which the
+parity tests hold to the oracle)."""
+import os
+import subprocess
+import sys
+
+import numpy as np
+import pytest
+
+from paper_1501_03869_gb300 import BP, Plan, _lib, synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
+def _handle(shape, ns, nt, tile=128, mode="table"):
+    rng = np.random.default_rng([shape[0], shape[1], ns, nt])
+    dx = 0.2e-3
+    speed = (1500.0 + 900.0 * synth.smooth_field(shape, 4.0, rng)).astype(np.float32)
+    hi = (np.array(shape[::-1], dtype=float) - 1) * dx
+    sensors = np.zeros((ns, 3))
+    sensors[:, 0] = np.where(np.arange(ns) % 2, hi[0], 0.0)
+    sensors[:, 1] = (np.floor(rng.uniform(0.0, 1.0, ns) * (shape[0] - 2)) + 0.37) * dx  # off the nodes
+    dt = 1.2 * float(np.linalg.norm(hi)) / 1500.0 / nt
+    flags = _lib.PAT_FLAG_TILE_256 if tile == 256 else _lib.PAT_FLAG_TILE_128
+    if mode == "constant":
+        return BP.constant(1560.0, shape, dx, np.zeros(3), sensors, dt, nt, flags=flags)
+    return BP(speed, dx, np.zeros(3), sensors, dt, nt, flags=flags | _lib.PAT_FLAG_GPU_TABLE)
+
+
+def _set_weights(bp, ns):
+    normals = np.zeros((ns, 3))
+    normals[:, 0] = np.where(np.arange(ns) % 2, -1.0, 1.0)
+    bp.set_solid_angle(normals, np.full(ns, 0.2e-3), 2 * np.pi)
+
+
+def _signals(frames, ns, nt, dtype="f32", seed=1):
+    g = torch.Generator("cuda").manual_seed(seed)
+    x = torch.randn(frames, ns, nt, generator=g, device="cuda")
+    if dtype == "f32":
+        return x, None
+    sc = x.abs().amax(dim=2).contiguous()
+    return (x / sc[..., None]).to(torch.bfloat16 if dtype == "bf16" else torch.float16).contiguous(), sc
+
+
+def _same(a, b):
+    return torch.equal(a.view(torch.int32), b.view(torch.int32))
+
+
+def _check_plan(bps, frames, dtype="f32", **kw):
+    """Executes twice (the second replays the graph where there is one); returns the plan's facts."""
+    sig, sc = zip(*[_signals(f, b.n_sensors, b.n_samples, dtype, i) for i, (b, f) in enumerate(zip(bps, frames))])
+    sc = None if dtype == "f32" else list(sc)
+    want = [b.reconstruct(s, scales=None if sc is None else sc[i]) for i, (b, s) in enumerate(zip(bps, sig))]
+    plan = Plan(bps, frames, dtype=dtype, **kw)
+    for _ in range(2):
+        outs = [torch.full_like(w, 7.0) for w in want]
+        plan.execute(list(sig), outs, scales=sc)
+        plan.sync()
+        assert all(_same(o, w) for o, w in zip(outs, want))
+    info = plan.info
+    plan.close()
+    return info
+
+
+@pytest.mark.parametrize("kw", [{}, dict(graph=True), dict(autotune=True, graph=True)], ids=["plain", "graph", "tuned"])
+@pytest.mark.parametrize("tile,nt", [(128, 17000), (128, 20000), (256, 12000)])
+def test_long_windows_of_many_frames(tile, nt, kw):
+    """Windows of 1 800 to 2 900 rows: a 32-frame row of them fits no CTA."""
+    with _handle((72, 80), 12, nt, tile) as a, _handle((64, 64), 9, 901, tile) as b:
+        assert 1800 <= a.info["window"] <= 2900, a.info["window"]
+        info = _check_plan([a, b], [32, 48], **kw)
+        assert info["fb_mask"] & 32 == 0
