@@ -684,10 +684,15 @@ extern "C" pat_status pat_bp_autotune(pat_bp_t h, const void* signals_dev, pat_d
                                       pat_stream_t stream) {
   if (!h) return fail(PAT_ERR_INVALID, "NULL handle");
   std::lock_guard<std::mutex> lk(h->mu);
+  if (n_frames < 1 || n_frames > 65535) return fail(PAT_ERR_INVALID, "n_frames must be 1..65535");
+  if (dtype != PAT_F32 && dtype != PAT_BF16 && dtype != PAT_F16) return fail(PAT_ERR_INVALID, "dtype");
+  // the rows that reconstruct() settles on: it may take shorter ones where
+  // windows are long
+  int wst = 0;
+  const int FB = n_frames < kStagedMinFrames ? frames_per_group(n_frames)
+                                             : pick_config(h, n_frames, fmt_for(dtype), &wst).FB;
   pat_plan_t pl = nullptr;
-  pat_status st = plan_new(&h, &n_frames, 1, dtype, 0, false,
-                           n_frames < kStagedMinFrames ? frames_per_group(n_frames) : frames_per_unit(h, n_frames),
-                           &pl);
+  pat_status st = plan_new(&h, &n_frames, 1, dtype, 0, false, FB, &pl);
   if (st != PAT_OK) return st;
   const void* sig[1] = {signals_dev};
   const float* sc[1] = {scales_dev};

@@ -80,3 +80,16 @@ def test_long_windows_of_many_frames(tile, nt, kw):
         assert 1800 <= a.info["window"] <= 2900, a.info["window"]
         info = _check_plan([a, b], [32, 48], **kw)
         assert info["fb_mask"] & 32 == 0
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_autotune_where_reconstruct_falls_back(dtype):
+    """The tuner takes the frames per unit that reconstruct() settles on."""
+    with _handle((128, 136), 260, 30000) as bp:
+        # enough units for rows of 32 frames, of which no window fits a CTA
+        assert bp.info["n_tiles"] * bp.info["split"] >= 4 * 152 and bp.info["window"] > 1752
+        sig, sc = _signals(32, 260, 30000, dtype)
+        want = bp.reconstruct(sig, scales=sc)
+        bp.autotune(sig, scales=sc)
+        assert _same(bp.reconstruct(sig, scales=sc), want)
+        bp.sync()
