@@ -112,9 +112,13 @@ int class_window(pat_plan_t pl, const std::vector<int>& idx, int S) {
   return w;
 }
 
-// Frames per unit of every instance.  Rows of 32 or 16 frames whose longest
-// window does not fit a CTA (32 frames: 1 752 rows) are halved down to 8, which
-// hold windows of almost 7 000.
+// Frames per unit of every instance.  Rows of 32 or 16 frames are halved, down
+// to 8, for a class whose units (frame group, tile, segment) would not fill the
+// chip -- fewer than four per SM in rows of 32, one in rows of 16 -- and for an
+// instance whose longest window does not fit a CTA (32 frames: 1 752 rows; 8:
+// almost 7 000).  32 BF16 frames, launches alone: 6 100 pixels x 64 sensors 36
+// us in rows of 32 (0.3 units per SM), 23 of 16 (0.6), 26 of 8 (1.2); x 256
+// sensors 56, 49, 63; 15 000 pixels x 256 sensors 99, 89, 93.
 std::vector<int> choose_frames_per_unit(pat_plan_t pl) {
   std::vector<int> fbs;
   for (size_t i = 0; i < pl->hs.size(); ++i) fbs.push_back(instance_fb(pl, int(i)));
@@ -124,12 +128,16 @@ std::vector<int> choose_frames_per_unit(pat_plan_t pl) {
     for (size_t i = 0; i < fbs.size(); ++i)
       if (fbs[i] == FB) idx.push_back(int(i));
     if (idx.empty()) continue;
+    int64_t units = 0;
+    for (int i : idx)
+      units += int64_t((pl->frames[i] + FB - 1) / FB) * pl->hs[i]->n_tiles * pl->hs[i]->n_seg;
+    const bool fill = units >= int64_t(FB == 32 ? 4 : 1) * pl->n_sm;
     GatherConfig c = class_config(pl, idx, FB);
     c.S = 1;
     for (int i : idx) {
       const int w = stage_window(pl->hs[i], 1);
       int wst = w;
-      if (!fit_stages(c, w, w, size_t(pl->hs[0]->max_smem), &wst)) fbs[i] = FB / 2;
+      if (!fill || !fit_stages(c, w, w, size_t(pl->hs[0]->max_smem), &wst)) fbs[i] = FB / 2;
     }
   }
   return fbs;

@@ -93,3 +93,16 @@ def test_autotune_where_reconstruct_falls_back(dtype):
         bp.autotune(sig, scales=sc)
         assert _same(bp.reconstruct(sig, scales=sc), want)
         bp.sync()
+
+
+@pytest.mark.parametrize("kw", [{}, dict(graph=True), dict(autotune=True, graph=True)], ids=["plain", "graph", "tuned"])
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+def test_rows_follow_the_units_of_a_class(dtype, kw):
+    """32-frame rows only where their units fill the chip: a small instance
+    takes 8-frame rows alone, and the long ones beside enough others."""
+    with _handle((72, 80), 64, 301) as small, _handle((160, 160), 256, 401) as big, \
+            _handle((152, 160), 250, 399) as other:
+        assert small.info["n_tiles"] < 152
+        assert _check_plan([small], [32], dtype, **kw)["fb_mask"] == 8
+        assert _check_plan([small, big], [8, 32], dtype, **kw)["fb_mask"] == 8 | 32
+        assert _check_plan([small, big, other], [32, 32, 48], dtype, **kw)["fb_mask"] == 16 | 32
