@@ -386,12 +386,14 @@ pat_status refresh_graph(pat_plan_t pl) {
 }
 
 // Shapes chosen earlier in this process (and, with PAT_TUNE_CACHE set, in a
-// text file of "signature S budget_kb" lines), keyed by the plan's shape.
+// text file of "signature S budget_kb" lines), keyed by the plan's shape.  The
+// signature starts with the version of the kernels that the shapes were timed
+// on; it changes whenever a shape means something else to them.
 std::mutex g_tune_mu;
 std::map<std::string, std::vector<int>> g_tune;
 
 std::string signature(pat_plan_t pl) {
-  std::string s = "sm" + std::to_string(pl->n_sm) + ".dt" + std::to_string(int(pl->dtype)) +
+  std::string s = "rows1.sm" + std::to_string(pl->n_sm) + ".dt" + std::to_string(int(pl->dtype)) +
                   ".fb" + std::to_string(pl->fb_uniform) + ".w" + std::to_string(pl->hs[0]->wgt) +
                   ".d" + std::to_string(pl->hs[0]->delays);
   for (size_t i = 0; i < pl->hs.size(); ++i) {
@@ -425,6 +427,13 @@ void tune_file_store(const std::string& key, int s, int b) {
   std::fclose(f);
 }
 
+// Shapes that tuning can choose: the classes' defaults (0, 0), or 4 to 32
+// sensors under a budget.
+bool known_shape(int S, int budget_kb) {
+  if (S == 0) return budget_kb == 0;
+  return (S == 4 || S == 8 || S == 16 || S == 32) && budget_kb > 0;
+}
+
 // Times every candidate shape (sensors per stage x shared-memory budget) on
 // the given inputs and keeps the fastest; the frames per unit of every
 // instance follow from its frame count.
@@ -434,11 +443,12 @@ pat_status autotune(pat_plan_t pl, const void* const* sig, const float* const* s
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     tune_file_load();
+    // a stored shape that is none of the candidates' kind or does not fit is tuned again
     auto it = g_tune.find(key);
-    if (it != g_tune.end()) {
-      pat_status s = plan_shape(pl, it->second[0], it->second[1]);
-      if (s == PAT_OK) pl->tuned = true;
-      return s;
+    if (it != g_tune.end() && known_shape(it->second[0], it->second[1]) &&
+        plan_shape(pl, it->second[0], it->second[1]) == PAT_OK) {
+      pl->tuned = true;
+      return PAT_OK;
     }
   }
   const int Ss[5] = {0, 4, 8, 16, 32};  // 0: the default shapes of the classes

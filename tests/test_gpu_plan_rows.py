@@ -106,3 +106,39 @@ def test_rows_follow_the_units_of_a_class(dtype, kw):
         assert _check_plan([small], [32], dtype, **kw)["fb_mask"] == 8
         assert _check_plan([small, big], [8, 32], dtype, **kw)["fb_mask"] == 8 | 32
         assert _check_plan([small, big, other], [32, 32, 48], dtype, **kw)["fb_mask"] == 16 | 32
+
+
+_TUNED = """
+import sys
+sys.path.insert(0, {root!r})
+sys.path.insert(0, {root!r} + "/tests")
+import test_gpu_plan_rows as t
+with t._handle((72, 80), 12, 9001) as a:
+    info = t._check_plan([a], [32], autotune=True, graph=True)
+    assert info["tuned"] == 1
+    print("ok", info["sensors_per_stage"], info["smem_budget_kb"], a.info["window"])
+"""
+
+
+def test_stored_shapes_that_do_not_fit(tmp_path):
+    """A stored launch shape of another kernel or one that holds no group is
+    tuned again, and a stored shape that fits is used."""
+    path = tmp_path / "shapes"
+
+    def run():
+        r = subprocess.run([sys.executable, "-c", _TUNED.format(root=ROOT)], capture_output=True, text=True,
+                           env=dict(os.environ, PAT_TUNE_CACHE=str(path)), timeout=300)
+        assert r.returncode == 0 and "ok" in r.stdout, r.stderr[-2000:]
+        return path.read_text().splitlines()
+
+    first = run()
+    assert len(first) == 1
+    key, s, b = first[0].split()
+    assert run() == first  # used, not tuned again
+    for bad in ("8 1", "24 200", "-4 100", "8 -5", "0 55", "64 200"):
+        path.write_text(f"{key} {bad}\n")
+        assert len(run()) == 2, bad
+    # as the staged kernel's shapes were stored
+    assert key.startswith("rows1.")
+    path.write_text(f"{key[len('rows1.'):]} 8 55\n")
+    assert len(run()) == 2
