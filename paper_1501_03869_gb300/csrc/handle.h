@@ -115,8 +115,8 @@ int stage_window(pat_bp_t h, int S);
 bool fit_stages(GatherConfig& c, int wmin, int wfull, size_t budget, int* wst);
 // launch shape: frames per unit, sensors per stage, stages under a smem budget
 GatherConfig config_for(pat_bp_t h, int n_frames, int FB, int S, size_t budget, int* wst);
-// (max_fb caps the frames per unit)
-GatherConfig pick_config(pat_bp_t h, int n_frames, int fmt, int* wst, int max_fb = 32);
+// (rows: frames per unit to start from, 0: frames_per_unit)
+GatherConfig pick_config(pat_bp_t h, int n_frames, int fmt, int* wst, int rows = 0);
 void default_shape(int FB, size_t limit, int* S, size_t* budget);
 // whole-tile or one-segment units for a launch of `tiles` (frame group, tile) pairs
 void set_units(GatherConfig& c, int64_t tiles, int n_seg);

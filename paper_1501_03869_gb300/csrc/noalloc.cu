@@ -76,7 +76,7 @@ extern "C" pat_status pat_bp_reconstruct_noalloc(pat_bp_t h, const void* signals
   const int fmt = fmt_for(dtype);
   int wst = 0;
   // at most 8 frames per unit: the scratch limit then admits what it always did
-  const GatherConfig c = pick_config(h, n_frames, fmt, &wst, 8);
+  const GatherConfig c = pick_config(h, n_frames, fmt, &wst, std::min(8, frames_per_unit(h, n_frames)));
   const int FB = c.FB;
   const size_t n_fg = size_t((n_frames + FB - 1) / FB);
 

@@ -548,7 +548,7 @@ void default_shape(int FB, size_t limit, int* S, size_t* budget) {
 // else frames per unit by count and the default shape.  When the windows are
 // too long for its budget, the budget grows to the device limit and then fewer
 // frames share a unit.  No choice here changes the summation order.
-GatherConfig pick_config(pat_bp_t h, int n_frames, int fmt, int* wst, int max_fb) {
+GatherConfig pick_config(pat_bp_t h, int n_frames, int fmt, int* wst, int rows) {
   const size_t limit = size_t(h->max_smem);
   if (n_frames < kStagedMinFrames && !(h->flags & PAT_FLAG_STAGED_SINGLE)) {
     // up to 3 frames: the unstaged kernels, one frame after the other (same
@@ -560,7 +560,7 @@ GatherConfig pick_config(pat_bp_t h, int n_frames, int fmt, int* wst, int max_fb
     c.no_window = (h->flags & PAT_FLAG_NO_WINDOW) != 0;
     return c;
   }
-  for (int FB = std::min(max_fb, frames_per_unit(h, n_frames)); FB >= 1; FB /= 2) {
+  for (int FB = rows ? rows : frames_per_unit(h, n_frames); FB >= 1; FB /= 2) {
     const int fi = fb_index(FB);
     int S = h->tuned_S[fi][fmt];
     size_t budget = size_t(h->tuned_budget_kb[fi][fmt]) * 1024;
@@ -811,7 +811,9 @@ static pat_status gather_locked(pat_bp_t h, int n_frames, float* out_dev, cudaSt
   if (n_frames < 1 || n_frames != h->pre_frames)
     return fail(PAT_ERR_INVALID, "gather needs the preprocess of the same n_frames first");
   int wst = 0;
-  const GatherConfig c = pick_config(h, n_frames, h->pre_fmt, &wst);
+  // the rows that the integrand lies in, also where the handle has got weights
+  // since and would now choose others
+  const GatherConfig c = pick_config(h, n_frames, h->pre_fmt, &wst, h->pre_fb);
   if (c.FB != h->pre_fb) return fail(PAT_ERR_INVALID, "frame grouping changed since preprocess");
   if (c.direct) {
     // one frame after the other, without the many-instance parameter block:

@@ -22,7 +22,7 @@ def _gpu():
         pytest.skip("no CUDA device")
 
 
-def _handle(shape, ns, nt, tile=128, mode="table"):
+def _handle(shape, ns, nt, tile=128, mode="table", weights=None):
     rng = np.random.default_rng([shape[0], shape[1], ns, nt])
     dx = 0.2e-3
     speed = (1500.0 + 900.0 * synth.smooth_field(shape, 4.0, rng)).astype(np.float32)
@@ -33,8 +33,8 @@ def _handle(shape, ns, nt, tile=128, mode="table"):
     dt = 1.2 * float(np.linalg.norm(hi)) / 1500.0 / nt
     flags = _lib.PAT_FLAG_TILE_256 if tile == 256 else _lib.PAT_FLAG_TILE_128
     if mode == "constant":
-        return BP.constant(1560.0, shape, dx, np.zeros(3), sensors, dt, nt, flags=flags)
-    return BP(speed, dx, np.zeros(3), sensors, dt, nt, flags=flags | _lib.PAT_FLAG_GPU_TABLE)
+        return BP.constant(1560.0, shape, dx, np.zeros(3), sensors, dt, nt, weights=weights, flags=flags)
+    return BP(speed, dx, np.zeros(3), sensors, dt, nt, weights=weights, flags=flags | _lib.PAT_FLAG_GPU_TABLE)
 
 
 def _set_weights(bp, ns):
@@ -142,3 +142,22 @@ def test_stored_shapes_that_do_not_fit(tmp_path):
     assert key.startswith("rows1.")
     path.write_text(f"{key[len('rows1.'):]} 8 55\n")
     assert len(run()) == 2
+
+
+@pytest.mark.parametrize("frames", [12, 48])
+def test_weights_set_between_preprocess_and_gather(frames):
+    """The gather takes the rows that preprocess() laid out, whatever rows the
+    handle's new mode would choose.  Sensor weights of one: preprocess() puts
+    the weights of its time into the multipliers."""
+    ones = np.ones(70, dtype=np.float32)
+    with _handle((256, 256), 70, 401, mode="constant", weights=ones) as bp, \
+            _handle((256, 256), 70, 401, mode="constant") as ref:
+        sig, _ = _signals(frames, 70, 401)
+        _set_weights(ref, 70)
+        want = ref.reconstruct(sig)
+        bp.preprocess(sig)
+        _set_weights(bp, 70)
+        out = torch.empty_like(want)
+        bp.gather(frames, out)
+        bp.sync()
+        assert _same(out, want)
