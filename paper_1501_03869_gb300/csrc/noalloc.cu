@@ -75,14 +75,15 @@ extern "C" pat_status pat_bp_reconstruct_noalloc(pat_bp_t h, const void* signals
   PAT_CUDA(cudaSetDevice(h->device));
   const int fmt = fmt_for(dtype);
   int wst = 0;
-  // at most 8 frames per unit: the scratch limit then admits what it always did
+  // at most 8 frames per unit, and no counters where rows of 4 frames and more
+  // take none: shorter rows then never need more scratch than rows of 8
   const GatherConfig c = pick_config(h, n_frames, fmt, &wst, std::min(8, frames_per_unit(h, n_frames)));
   const int FB = c.FB;
   const size_t n_fg = size_t((n_frames + FB - 1) / FB);
 
   // scratch layout: unit tickets | segment counters | partials | multipliers | integrand
   const size_t sched_bytes = 256;
-  const size_t cnt_bytes = align256(n_fg * h->n_tiles * sizeof(int));
+  const size_t cnt_bytes = FB >= 4 ? 0 : align256(n_fg * h->n_tiles * sizeof(int));
   const size_t part_bytes =
       align256(n_fg * h->n_tiles * h->n_seg * std::max(FB, h->SW) * h->P * sizeof(float));
   const size_t m_bytes = align256(n_fg * h->ns_pad * FB * sizeof(float));
@@ -100,7 +101,8 @@ extern "C" pat_status pat_bp_reconstruct_noalloc(pat_bp_t h, const void* signals
   float* part = reinterpret_cast<float*>(base + sched_bytes + cnt_bytes);
   float* m = reinterpret_cast<float*>(base + sched_bytes + cnt_bytes + part_bytes);
   void* b = base + sched_bytes + cnt_bytes + part_bytes + m_bytes;
-  // what must start at zero: the unit tickets and the segment counters
+  // what must start at zero: the unit tickets and the segment counters (rows of
+  // 1 and 2 frames)
   PAT_CUDA(cudaMemsetAsync(base, 0, sched_bytes + cnt_bytes, stream));
 
   PreParams pp = make_pre(h, signals_dev, dtype, scales_dev, n_frames, FB);

@@ -161,3 +161,20 @@ def test_weights_set_between_preprocess_and_gather(frames):
         bp.gather(frames, out)
         bp.sync()
         assert _same(out, want)
+
+
+def test_noalloc_at_the_scratch_limit():
+    """32 frames that need exactly the 16 MiB in rows of 8: 36 tiles, 50 sensors,
+    2 528 padded samples.  The launch takes rows of 4 (36 tiles fill no chip),
+    which must not need more."""
+    with _handle((64, 72), 50, 2527) as bp:
+        assert bp.info["n_tiles"] == 36 and bp.info["n_samples_pad"] == 2528 and bp.info["tile_pix"] == 128
+        sig, _ = _signals(32, 50, 2527)
+        want = bp.reconstruct(sig)
+        out = torch.full_like(want, 7.0)
+        bp.reconstruct_noalloc(sig, out)
+        bp.sync()
+        assert _same(out, want)
+        more, _ = _signals(33, 50, 2527)
+        with pytest.raises(Exception, match="scratch"):
+            bp.reconstruct_noalloc(more, torch.empty(bp.out_shape(33), device="cuda"))
