@@ -109,15 +109,19 @@ int fb_index(int FB);
 int fmt_for(pat_dtype dt);
 // device buffers for n_frames frames grouped by FB (grown, zero-filled)
 pat_status ensure_buffers_fb(pat_bp_t h, int n_frames, int FB);
+// buffers of any launch of at most n_frames frames
+pat_status reserve_frames(pat_bp_t h, int n_frames);
 // window rows one pipeline stage of S sensors can need
 int stage_window(pat_bp_t h, int S);
 // stages and window-row budget of a shape under a smem budget (false: nothing fits)
 bool fit_stages(GatherConfig& c, int wmin, int wfull, size_t budget, int* wst);
 // launch shape: frames per unit, sensors per stage, stages under a smem budget
-GatherConfig config_for(pat_bp_t h, int n_frames, int FB, int S, size_t budget, int* wst);
-// (rows: frames per unit to start from, 0: frames_per_unit)
-GatherConfig pick_config(pat_bp_t h, int n_frames, int fmt, int* wst, int rows = 0);
+GatherConfig config_for(pat_bp_t h, int n_frames, int FB, int S, size_t budget, int* wst, bool* fits = nullptr);
+// (rows: frames per unit to start from, 0: frames_per_unit; lean: for a scratch limit)
+GatherConfig pick_config(pat_bp_t h, int n_frames, int fmt, int* wst, int rows = 0, bool lean = false);
 void default_shape(int FB, size_t limit, int* S, size_t* budget);
+// batched gather: shared memory besides the ring, and bytes of the longest window
+void ring_need(GatherConfig c, int longest, size_t* fixed, size_t* window);
 // whole-tile or one-segment units for a launch of `tiles` (frame group, tile) pairs
 void set_units(GatherConfig& c, int64_t tiles, int n_seg);
 // units of one instance

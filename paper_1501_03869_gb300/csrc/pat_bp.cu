@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "handle.h"
+#include "row_rules.h"
 
 using namespace patbp;
 
@@ -447,6 +448,16 @@ pat_status ensure_buffers_fb(pat_bp_t h, int n_frames, int FB) {
   return PAT_OK;
 }
 
+// Buffers of any launch of at most n_frames frames: the longest rows need the
+// most frame slots, single frames (long windows) the most partial sums.
+pat_status reserve_frames(pat_bp_t h, int n_frames) {
+  const pat_status st = ensure_buffers_fb(h, n_frames, frames_per_group(n_frames));
+  if (st != PAT_OK || n_frames < kStagedMinFrames) return st;
+  int wst = 0;
+  const int FB = pick_config(h, n_frames, kBF32, &wst).FB;
+  return FB < 4 ? ensure_buffers_fb(h, n_frames, FB) : PAT_OK;
+}
+
 // Largest sum of window lengths over the S-sensor stages of any tile: the
 // window rows one pipeline stage must hold.
 int stage_window(pat_bp_t h, int S) {
@@ -508,7 +519,7 @@ bool fit_stages(GatherConfig& c, int wmin, int wfull, size_t budget, int* wst) {
 
 // Launch shape under a shared-memory budget: stages and row budget as
 // fit_stages decides; fewer sensors per stage if nothing fits.
-GatherConfig config_for(pat_bp_t h, int n_frames, int FB, int S, size_t budget, int* wst) {
+GatherConfig config_for(pat_bp_t h, int n_frames, int FB, int S, size_t budget, int* wst, bool* fits) {
   GatherConfig c;
   c.P = h->P;
   c.SW = h->SW;
@@ -521,7 +532,9 @@ GatherConfig config_for(pat_bp_t h, int n_frames, int FB, int S, size_t budget, 
   const int wmin = stage_window(h, 1);
   if (FB >= 4) c.S = std::min(S, 16);
   for (;;) {
-    if (fit_stages(c, wmin, stage_window(h, c.S), budget, wst)) break;
+    const bool ok = fit_stages(c, wmin, stage_window(h, c.S), budget, wst);
+    if (fits) *fits = ok;
+    if (ok) break;
     if (FB >= 4 && c.S > 1) {
       c.S /= 2;
       continue;
@@ -530,6 +543,14 @@ GatherConfig config_for(pat_bp_t h, int n_frames, int FB, int S, size_t budget, 
     c.S /= 2;
   }
   return c;
+}
+
+// (The same for every mode of a handle, so that its rows do not change with its
+// weights; delay data and multipliers are small beside windows that matter.)
+void ring_need(GatherConfig c, int longest, size_t* fixed, size_t* window) {
+  c.ring = 0;
+  *fixed = gather_smem_bytes(c, 0);
+  *window = size_t(longest) * c.FB * 4;
 }
 
 // Sensors per group (stage) and shared-memory budget of an untuned launch.
@@ -545,10 +566,12 @@ void default_shape(int FB, size_t limit, int* S, size_t* budget) {
 }
 
 // Launch shape for a frame count: the autotuned one when the handle has it,
-// else frames per unit by count and the default shape.  When the windows are
-// too long for its budget, the budget grows to the device limit and then fewer
-// frames share a unit.  No choice here changes the summation order.
-GatherConfig pick_config(pat_bp_t h, int n_frames, int fmt, int* wst, int rows) {
+// else frames per unit by count and the default shape, with a larger budget
+// where windows are long.  Rows too long for the windows are halved, and rows of
+// 4 give way to single frames (lean: to pairs, and only where two windows and a
+// pipeline of 16 KB do not fit, since single frames hold four partial sums per
+// pixel instead of one).  No choice here changes the summation order.
+GatherConfig pick_config(pat_bp_t h, int n_frames, int fmt, int* wst, int rows, bool lean) {
   const size_t limit = size_t(h->max_smem);
   if (n_frames < kStagedMinFrames && !(h->flags & PAT_FLAG_STAGED_SINGLE)) {
     // up to 3 frames: the unstaged kernels, one frame after the other (same
@@ -564,8 +587,31 @@ GatherConfig pick_config(pat_bp_t h, int n_frames, int fmt, int* wst, int rows) 
     const int fi = fb_index(FB);
     int S = h->tuned_S[fi][fmt];
     size_t budget = size_t(h->tuned_budget_kb[fi][fmt]) * 1024;
-    if (S <= 0) default_shape(FB, limit, &S, &budget);
-    GatherConfig c = config_for(h, n_frames, FB, S, budget, wst);
+    const bool tuned = S > 0;
+    if (!tuned) default_shape(FB, limit, &S, &budget);
+    GatherConfig c;
+    if (FB >= 4) {
+      size_t fixed = 0, window = 0;
+      c = config_for(h, n_frames, FB, 1, limit, wst);
+      ring_need(c, stage_window(h, 1), &fixed, &window);
+      if (!ring_is_deep(FB, fixed, window, limit) &&
+          !(lean && FB == 4 && fixed + 2 * window + 16 * 1024 <= limit))
+        continue;
+      bool fits = false;
+      if (tuned) c = config_for(h, n_frames, FB, S, budget, wst, &fits);
+      if (fits) return c;
+      if (tuned) default_shape(FB, limit, &S, &budget);
+      return config_for(h, n_frames, FB, S, ring_budget(budget, fixed, window, FB, limit), wst);
+    }
+    if (n_frames >= kStagedMinFrames && !lean) {
+      // long windows: single frames; all of the SM where it gets few units (4
+      // frames of 8 700 pixels x 96 sensors, windows of 3 280 rows, 3.6 units
+      // per SM: 37 us, 49 in 72 KB; 32 frames, 29 per SM: 149 in 72 KB and, with
+      // 3 736 rows, 168 against 196)
+      if (FB == 2) continue;
+      if (!tuned && int64_t(n_frames) * h->n_tiles * h->n_seg < int64_t(20) * h->n_sm) budget = limit;
+    }
+    c = config_for(h, n_frames, FB, S, budget, wst);
     if (gather_smem_bytes(c, *wst) <= limit) return c;
     c = config_for(h, n_frames, FB, 8, limit, wst);  // longer windows: the whole SM
     if (gather_smem_bytes(c, *wst) <= limit) return c;
@@ -772,16 +818,13 @@ extern "C" pat_status pat_bp_restore(pat_bp_t h, pat_stream_t stream) {
   return restore_locked(h, static_cast<cudaStream_t>(stream));
 }
 
-static pat_status ensure_buffers(pat_bp_t h, int n_frames) {
-  return ensure_buffers_fb(h, n_frames, frames_per_group(n_frames));
-}
 
 extern "C" pat_status pat_bp_reserve(pat_bp_t h, int max_frames, pat_dtype dtype) {
   if (!h || max_frames < 1) return fail(PAT_ERR_INVALID, "bad handle or frame count");
   (void)dtype;
   std::lock_guard<std::mutex> lk(h->mu);
   PAT_CUDA(cudaSetDevice(h->device));
-  return ensure_buffers(h, max_frames);
+  return reserve_frames(h, max_frames);
 }
 
 static pat_status preprocess_locked(pat_bp_t h, const void* signals_dev, pat_dtype dtype,

@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "handle.h"
+#include "row_rules.h"
 
 using namespace patbp;
 
@@ -115,10 +116,10 @@ int class_window(pat_plan_t pl, const std::vector<int>& idx, int S) {
 // Frames per unit of every instance.  Rows of 32 or 16 frames are halved, down
 // to 8, for a class whose units (frame group, tile, segment) would not fill the
 // chip -- fewer than four per SM in rows of 32, one in rows of 16 -- and for an
-// instance whose longest window does not fit a CTA (32 frames: 1 752 rows; 8:
-// almost 7 000).  32 BF16 frames, launches alone: 6 100 pixels x 64 sensors 36
-// us in rows of 32 (0.3 units per SM), 23 of 16 (0.6), 26 of 8 (1.2); x 256
-// sensors 56, 49, 63; 15 000 pixels x 256 sensors 99, 89, 93.
+// instance whose windows are too long for them.  32 BF16 frames, launches
+// alone: 6 100 pixels x 64 sensors 36 us in rows of 32 (0.3 units per SM), 23 of
+// 16 (0.6), 26 of 8 (1.2); x 256 sensors 56, 49, 63; 15 000 pixels x 256 sensors
+// 99, 89, 93.
 std::vector<int> choose_frames_per_unit(pat_plan_t pl) {
   std::vector<int> fbs;
   for (size_t i = 0; i < pl->hs.size(); ++i) fbs.push_back(instance_fb(pl, int(i)));
@@ -132,12 +133,11 @@ std::vector<int> choose_frames_per_unit(pat_plan_t pl) {
     for (int i : idx)
       units += int64_t((pl->frames[i] + FB - 1) / FB) * pl->hs[i]->n_tiles * pl->hs[i]->n_seg;
     const bool fill = units >= int64_t(FB == 32 ? 4 : 1) * pl->n_sm;
-    GatherConfig c = class_config(pl, idx, FB);
-    c.S = 1;
+    const GatherConfig c = class_config(pl, idx, FB);
     for (int i : idx) {
-      const int w = stage_window(pl->hs[i], 1);
-      int wst = w;
-      if (!fill || !fit_stages(c, w, w, size_t(pl->hs[0]->max_smem), &wst)) fbs[i] = FB / 2;
+      size_t fixed = 0, window = 0;
+      ring_need(c, stage_window(pl->hs[i], 1), &fixed, &window);
+      if (!fill || !ring_is_deep(FB, fixed, window, size_t(pl->hs[0]->max_smem))) fbs[i] = FB / 2;
     }
   }
   return fbs;
@@ -163,17 +163,22 @@ pat_status plan_shape(pat_plan_t pl, int S, int budget_kb) {
   for (PlanClass& k : cls) {
     int Sk = S;
     size_t budget = std::min(size_t(budget_kb) * 1024, limit);
+    GatherConfig c = class_config(pl, k.idx, k.FB);
+    const int wmin = class_window(pl, k.idx, 1);
     if (S == 0) {
       default_shape(k.FB, limit, &Sk, &budget);
+      if (k.FB >= 4) {
+        size_t fixed = 0, window = 0;
+        ring_need(c, wmin, &fixed, &window);
+        budget = ring_budget(budget, fixed, window, k.FB, limit);
+      }
       pl->S = std::max(pl->S, Sk);
       pl->budget_kb = std::max(pl->budget_kb, int(budget / 1024));
     }
     if (k.FB >= 4) Sk = std::min(Sk, 16);
     // one shape per class: the longest single window and the longest
     // S-sensor window sum of its instances bound the stages' row budget
-    const int wmin = class_window(pl, k.idx, 1);
     int wfull = class_window(pl, k.idx, Sk);
-    GatherConfig c = class_config(pl, k.idx, k.FB);
     c.S = Sk;
     int wst = wfull;
     bool fits = fit_stages(c, wmin, wfull, budget, &wst);

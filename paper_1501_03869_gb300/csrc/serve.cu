@@ -200,7 +200,7 @@ void reap(pat_srv_t s, std::unique_lock<std::mutex>& lk) {
 // every smaller batch too (n frames in groups of FB take at most as much).
 pat_status reserve_batch_buffers(pat_srv_t s, pat_bp_t h) {
   const int F = s->cfg.max_batch_frames;
-  return ensure_buffers_fb(h, F, frames_per_group(F));
+  return reserve_frames(h, F);
 }
 
 // Make subject k resident within the budget, evicting least recently used idle

@@ -178,3 +178,38 @@ def test_noalloc_at_the_scratch_limit():
         more, _ = _signals(33, 50, 2527)
         with pytest.raises(Exception, match="scratch"):
             bp.reconstruct_noalloc(more, torch.empty(bp.out_shape(33), device="cuda"))
+
+
+@pytest.mark.parametrize("frames,nt,budget", [(8, 2001, 72), (8, 6001, 110), (8, 9001, 200), (5, 6001, 110)])
+def test_plans_widen_the_ring_for_long_windows(frames, nt, budget):
+    """Windows of 240, 712 and 1 072 rows of 8 frames, 712 of 4: the budget
+    grows before a ring gets down to one group."""
+    with _handle((72, 80), 12, nt) as bp:
+        info = _check_plan([bp], [frames])
+        kb = info["smem_budget_kb"]
+        assert kb == budget if budget < 200 else kb >= budget, (kb, bp.info["window"])
+
+
+@pytest.mark.parametrize("frames", [4, 16, 23, 32])
+@pytest.mark.parametrize("nt", [9001, 17000, 26000, 32000])
+def test_reserved_handle_allocates_nothing_for_long_windows(frames, nt):
+    """1 072 to 3 912 rows per window: rows of 16 down to single frames, whose
+    partial sums take the most; every frame as through the kernels for one
+    frame, first under capture, then through the no-allocation path."""
+    with _handle((72, 80), 12, nt) as bp, _handle((72, 80), 12, nt) as ref:
+        sig, _ = _signals(frames, 12, nt)
+        want = torch.cat([ref.reconstruct(sig[f:f + 1]) for f in range(frames)])
+        bp.reserve(32)
+        out = torch.empty_like(want)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            bp.reconstruct(sig, out=out)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert _same(out, want)
+        few = sig[:4]
+        out = torch.full_like(want[:4], 7.0)
+        bp.reconstruct_noalloc(few, out)
+        bp.sync()
+        assert _same(out, want[:4])
