@@ -44,11 +44,15 @@
 namespace patbp {
 
 // ------------------------------------------------------------------ shape --
-template <int P, int FB, int FMT>
+template <int P, int FB, int FMT, int MODE>
 struct RowsShape {
   // 16-byte quads of a row that a lane owns: two where the two loads can be
-  // kept free of bank conflicts (halves the index work per update)
-  static constexpr int NQ = FB == 32 || (FB == 16 && FMT == kBF32) ? 2 : 1;
+  // kept free of bank conflicts (halves the index work per update), and in
+  // 8-frame rows where offsets or weights are computed, whose arithmetic then
+  // stays in one lane without shuffles (24 FP32 frames of 22 300 pixels x 512
+  // sensors, constant speed with weights: 294 -> 259 us, 256-pixel tiles 263 ->
+  // 222; stored delays are faster with one, 198 us against 201).
+  static constexpr int NQ = FB == 32 || (FB == 16 && FMT == kBF32) || (FB == 8 && MODE != 0) ? 2 : 1;
   static constexpr int LPP = FB / (4 * NQ);               // lanes that share a pixel
   static constexpr int PPW = 32 / LPP;                    // pixels of one warp-wide load
   static constexpr int NW = FB >= 16 ? 8 : 4;             // consumer warps
@@ -57,8 +61,12 @@ struct RowsShape {
   static constexpr int A = NPX / PPW;                     // pixels of a lane
   static constexpr int V = A < 4 ? A : (NQ == 2 ? 4 : 2); // of which neighbours in the tile
   static constexpr int THREADS = 32 * (NW + 1 + NC);
-  // resident CTAs per SM the registers must allow: 11 to 18 warps
-  static constexpr int MIN_CTAS = FB >= 16 ? 1 : 3;
+  // resident CTAs per SM the registers must allow: 11 to 18 warps.  8-frame rows
+  // spill in the 96 registers of three where a lane owns four pixels (256-pixel
+  // tiles) or computes offsets or weights: two are faster there (24 FP32 frames
+  // as above, 256-pixel tiles 184 -> 166 us; 12 frames of 6 600 pixels x 128
+  // sensors, constant speed 34 -> 28 us, with weights too 39 -> 31).
+  static constexpr int MIN_CTAS = FB >= 16 ? 1 : (FB == 8 && (P == 256 || MODE != 0) ? 2 : 3);
   static_assert(A % V == 0 && NPX * NW == P, "pixels of a lane");
 };
 
@@ -84,9 +92,9 @@ __device__ __forceinline__ RowsUnit decode_rows(const StreamParams& p, int64_t u
 }
 
 template <int P, int FB, int FMT, int SW, int MODE>
-__global__ void __launch_bounds__(RowsShape<P, FB, FMT>::THREADS, RowsShape<P, FB, FMT>::MIN_CTAS)
+__global__ void __launch_bounds__(RowsShape<P, FB, FMT, MODE>::THREADS, RowsShape<P, FB, FMT, MODE>::MIN_CTAS)
     gather_rows_kernel(const __grid_constant__ StreamParams p) {
-  using SH = RowsShape<P, FB, FMT>;
+  using SH = RowsShape<P, FB, FMT, MODE>;
   constexpr int DELAYS = MODE & 1, WGT = (MODE >> 1) & 1;
   constexpr int A = SH::A, V = SH::V, NQ = SH::NQ, LPP = SH::LPP, PPW = SH::PPW, NPX = SH::NPX, NW = SH::NW;
   constexpr int NC = SH::NC;
@@ -731,7 +739,7 @@ __global__ void __launch_bounds__(256) rows_reduce_kernel(const __grid_constant_
 template <int P, int FB, int FMT, int SW, int MODE>
 static cudaError_t rows_t(const StreamParams& p, size_t smem, int grid, cudaStream_t st, int* resident,
                           int n_sm) {
-  using SH = RowsShape<P, FB, FMT>;
+  using SH = RowsShape<P, FB, FMT, MODE>;
   auto kern = gather_rows_kernel<P, FB, FMT, SW, MODE>;
   static SmemGrant grant;
   if (cudaError_t e = grant_smem(grant, kern, smem); e != cudaSuccess) return e;

@@ -104,7 +104,9 @@ namespace patbp {
 constexpr int kStagedMinFrames = 4;
 int frames_per_group(int n_frames);
 // frames per unit that suit a handle's reconstruction of n_frames (1 below kStagedMinFrames)
-int frames_per_unit(pat_bp_t h, int n_frames);
+int frames_per_unit(pat_bp_t h, int n_frames, int fmt);
+// whether rows of FB frames suit the delays and the integrand's format
+bool rows_suit(int FB, int delays, int fmt);
 int fb_index(int FB);
 int fmt_for(pat_dtype dt);
 // device buffers for n_frames frames grouped by FB (grown, zero-filled)
@@ -119,7 +121,7 @@ bool fit_stages(GatherConfig& c, int wmin, int wfull, size_t budget, int* wst);
 GatherConfig config_for(pat_bp_t h, int n_frames, int FB, int S, size_t budget, int* wst, bool* fits = nullptr);
 // (rows: frames per unit to start from, 0: frames_per_unit; lean: for a scratch limit)
 GatherConfig pick_config(pat_bp_t h, int n_frames, int fmt, int* wst, int rows = 0, bool lean = false);
-void default_shape(int FB, size_t limit, int* S, size_t* budget);
+void default_shape(const GatherConfig& c, size_t limit, int* S, size_t* budget);
 // batched gather: shared memory besides the ring, and bytes of the longest window
 void ring_need(GatherConfig c, int longest, size_t* fixed, size_t* window);
 // whole-tile or one-segment units for a launch of `tiles` (frame group, tile) pairs

@@ -77,7 +77,7 @@ extern "C" pat_status pat_bp_reconstruct_noalloc(pat_bp_t h, const void* signals
   int wst = 0;
   // at most 8 frames per unit, and no counters where rows of 4 frames and more
   // take none: shorter rows then never need more scratch than rows of 8
-  const GatherConfig c = pick_config(h, n_frames, fmt, &wst, std::min(8, frames_per_unit(h, n_frames)), true);
+  const GatherConfig c = pick_config(h, n_frames, fmt, &wst, std::min(8, frames_per_unit(h, n_frames, fmt)), true);
   const int FB = c.FB;
   const size_t n_fg = size_t((n_frames + FB - 1) / FB);
 

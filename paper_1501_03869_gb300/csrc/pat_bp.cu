@@ -377,23 +377,27 @@ int frames_per_group(int n_frames) {
   return n_frames >= 8 ? 8 : (n_frames >= 4 ? 4 : (n_frames >= 2 ? 2 : 1));
 }
 
-int frames_per_unit(pat_bp_t h, int n_frames) {
+int frames_per_unit(pat_bp_t h, int n_frames, int fmt) {
   if (n_frames < kStagedMinFrames && !(h->flags & PAT_FLAG_STAGED_SINGLE)) return 1;
   // Long rows make few units: shorter ones where the launch would have fewer
   // than four units per SM (8-frame rows: one), down to 4 frames.  64 BF16
   // frames of 6 092 pixels x 64 sensors: 41 us in rows of 32 (96 units), 34 of
   // 16, 32 of 8, 43 of 4; 5 000 pixels x 256 sensors: 157, 121, 139, 125.
   int FB = frames_per_group(n_frames);
-  // computed delays and weights together outweigh what 16-frame rows save (12
-  // FP16 frames: 181 us in rows of 16, 174 of 8)
-  if (h->delays && h->wgt && h->P == 128 && FB == 16) FB = 8;
   while (FB > 4) {
     const int64_t units = int64_t((n_frames + FB - 1) / FB) * h->n_tiles * h->n_seg;
-    if (units >= int64_t(FB == 8 ? 1 : 4) * h->n_sm) break;
+    if (units >= int64_t(FB == 8 ? 1 : 4) * h->n_sm && rows_suit(FB, h->delays, fmt)) break;
     FB /= 2;
   }
   return FB;
 }
+
+// A lane of a 16-bit row of 16 frames owns a quarter of a pixel's frames and
+// computes its offset for them alone: with computed delays rows of 8 are faster
+// (12 FP16 frames of 22 300 pixels x 512 sensors: 151 us, 168 in rows of 16;
+// with weights 168 and 195; FP32 owns half and prefers 16, 157 against 163 and
+// 169 against 180).
+bool rows_suit(int FB, int delays, int fmt) { return !(FB == 16 && delays && fmt != kBF32); }
 
 int fb_index(int FB) {
   int i = 0;
@@ -557,12 +561,17 @@ void ring_need(GatherConfig c, int longest, size_t* fixed, size_t* window) {
 // Batched gather, measured on 152 SMs: rows of 16 and 32 frames take the whole
 // SM (one CTA of 8 consumer warps; half the ring is 1.2 to 1.8 times slower),
 // 8-frame rows three CTAs of 4 consumer warps (8 frames of 1.04 M voxels,
-// BF16: 2.12 ms; two CTAs 2.60, four 2.41).
-void default_shape(int FB, size_t limit, int* S, size_t* budget) {
+// BF16: 2.12 ms; two CTAs 2.60, four 2.41) or the two that their registers allow
+// (24 FP32 frames of 22 300 pixels x 512 sensors, 256-pixel tiles: 166 us in 110
+// KB, 184 in 72), groups of 8 sensors where 128-pixel tiles compute offsets or
+// weights (8 frames of 0.3 M voxels x 256 sensors, weights: 351 us, 458 in groups
+// of 4).
+void default_shape(const GatherConfig& c, size_t limit, int* S, size_t* budget) {
   static const int s[6] = {16, 8, 8, 4, 8, 4}, kb[6] = {72, 100, 72, 72, 0, 0};
-  const int i = fb_index(FB);
-  *S = s[i];
-  *budget = kb[i] ? size_t(kb[i]) * 1024 : limit;
+  const int i = fb_index(c.FB);
+  const bool mode = c.delays || c.wgt;
+  *S = c.FB == 8 && c.P == 128 && mode ? 8 : s[i];
+  *budget = kb[i] ? size_t(c.FB == 8 && (c.P == 256 || mode) ? 110 : kb[i]) * 1024 : limit;
 }
 
 // Launch shape for a frame count: the autotuned one when the handle has it,
@@ -583,16 +592,15 @@ GatherConfig pick_config(pat_bp_t h, int n_frames, int fmt, int* wst, int rows, 
     c.no_window = (h->flags & PAT_FLAG_NO_WINDOW) != 0;
     return c;
   }
-  for (int FB = rows ? rows : frames_per_unit(h, n_frames); FB >= 1; FB /= 2) {
+  for (int FB = rows ? rows : frames_per_unit(h, n_frames, fmt); FB >= 1; FB /= 2) {
     const int fi = fb_index(FB);
     int S = h->tuned_S[fi][fmt];
     size_t budget = size_t(h->tuned_budget_kb[fi][fmt]) * 1024;
     const bool tuned = S > 0;
-    if (!tuned) default_shape(FB, limit, &S, &budget);
-    GatherConfig c;
+    GatherConfig c = config_for(h, n_frames, FB, 1, limit, wst);
+    if (!tuned) default_shape(c, limit, &S, &budget);
     if (FB >= 4) {
       size_t fixed = 0, window = 0;
-      c = config_for(h, n_frames, FB, 1, limit, wst);
       ring_need(c, stage_window(h, 1), &fixed, &window);
       if (!ring_is_deep(FB, fixed, window, limit) &&
           !(lean && FB == 4 && fixed + 2 * window + 16 * 1024 <= limit))
@@ -600,7 +608,7 @@ GatherConfig pick_config(pat_bp_t h, int n_frames, int fmt, int* wst, int rows, 
       bool fits = false;
       if (tuned) c = config_for(h, n_frames, FB, S, budget, wst, &fits);
       if (fits) return c;
-      if (tuned) default_shape(FB, limit, &S, &budget);
+      if (tuned) default_shape(c, limit, &S, &budget);
       return config_for(h, n_frames, FB, S, ring_budget(budget, fixed, window, FB, limit), wst);
     }
     if (n_frames >= kStagedMinFrames && !lean) {

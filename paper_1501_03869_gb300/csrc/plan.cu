@@ -132,8 +132,8 @@ std::vector<int> choose_frames_per_unit(pat_plan_t pl) {
     int64_t units = 0;
     for (int i : idx)
       units += int64_t((pl->frames[i] + FB - 1) / FB) * pl->hs[i]->n_tiles * pl->hs[i]->n_seg;
-    const bool fill = units >= int64_t(FB == 32 ? 4 : 1) * pl->n_sm;
     const GatherConfig c = class_config(pl, idx, FB);
+    const bool fill = units >= int64_t(FB == 32 ? 4 : 1) * pl->n_sm && rows_suit(FB, c.delays, pl->fmt);
     for (int i : idx) {
       size_t fixed = 0, window = 0;
       ring_need(c, stage_window(pl->hs[i], 1), &fixed, &window);
@@ -166,7 +166,7 @@ pat_status plan_shape(pat_plan_t pl, int S, int budget_kb) {
     GatherConfig c = class_config(pl, k.idx, k.FB);
     const int wmin = class_window(pl, k.idx, 1);
     if (S == 0) {
-      default_shape(k.FB, limit, &Sk, &budget);
+      default_shape(c, limit, &Sk, &budget);
       if (k.FB >= 4) {
         size_t fixed = 0, window = 0;
         ring_need(c, wmin, &fixed, &window);

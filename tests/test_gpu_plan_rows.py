@@ -213,3 +213,20 @@ def test_reserved_handle_allocates_nothing_for_long_windows(frames, nt):
         bp.reconstruct_noalloc(few, out)
         bp.sync()
         assert _same(out, want[:4])
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("tile", [128, 256])
+def test_shapes_of_computed_delays(tile, dtype):
+    """Constant speed: 16-bit frames take rows of 8 where FP32 takes 16, and
+    8-frame rows get the shared memory of two CTAs per SM, whose registers hold
+    what three would spill; stored delays of 128-pixel tiles keep three."""
+    with _handle((160, 160), 256, 401, tile, "constant") as bp, _handle((160, 160), 256, 401, tile) as table:
+        assert _check_plan([bp], [48], dtype)["fb_mask"] == (16 if dtype == "f32" else 8)
+        info = _check_plan([bp], [8], dtype)
+        assert info["smem_budget_kb"] == 110 and info["sensors_per_stage"] == (8 if tile == 128 else 4)
+        info = _check_plan([table], [8], dtype)
+        assert info["smem_budget_kb"] == (72 if tile == 128 else 110)
+        _set_weights(bp, 256)
+        assert _check_plan([bp], [48], dtype)["fb_mask"] == (16 if dtype == "f32" else 8)
+        assert _check_plan([bp], [24], dtype)["smem_budget_kb"] == 110
