@@ -374,8 +374,12 @@ bool layout_pixels(const GridDesc& g, const uint8_t* mask, int P, bool compact_o
       if (mask[v]) { ++v; continue; }
       int64_t s = v;
       while (v < total && !mask[v]) ++v;
-      out.zero_runs.push_back(int32_t(s));
-      out.zero_runs.push_back(int32_t(v - s));
+      // in pieces that warps share evenly: the rows above and below a small
+      // mask are one run of tens of thousands of nodes
+      for (int64_t at = s; at < v; at += kZeroRunMax) {
+        out.zero_runs.push_back(int32_t(at));
+        out.zero_runs.push_back(int32_t(std::min<int64_t>(kZeroRunMax, v - at)));
+      }
     }
   }
   return true;

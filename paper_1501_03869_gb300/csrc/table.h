@@ -36,6 +36,8 @@ struct GridDesc {
   int64_t total() const { return int64_t(n[0]) * n[1] * n[2]; }
 };
 
+constexpr int64_t kZeroRunMax = 512;  // nodes of one run to clear
+
 struct HostTable {
   int P = 0;
   int n_tiles = 0;
@@ -47,7 +49,7 @@ struct HostTable {
   std::vector<uint16_t> len;        // [n_tiles][n_sensors]
   std::vector<int32_t> slot_dense;  // [n_tiles * P] dense grid index or -1
   std::vector<int32_t> slot_compact;// [n_tiles * P] raster rank among mask pixels or -1
-  std::vector<int32_t> zero_runs;   // pairs (start, length) of non-mask runs of the grid
+  std::vector<int32_t> zero_runs;   // pairs (start, length <= kZeroRunMax) of non-mask runs of the grid
   // constant-speed delays (build_constant_layout): no u; instead
   std::vector<float> anchor;        // [n_tiles][n_sensors][8] per-sensor anchor of each tile
   std::vector<float> pixq;          // [n_tiles][P][4] per-pixel terms relative to the anchor

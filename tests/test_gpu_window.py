@@ -56,3 +56,31 @@ def test_windowed_equals_unwindowed(mode, tile, nt):
                 assert torch.equal(ia.view(torch.int32), ib.view(torch.int32)), (ns, dtype, a.info["window"])
             a.sync()
             b.sync()
+
+
+@pytest.mark.parametrize("imaged", ["few", "scattered", "none but one"])
+@pytest.mark.parametrize("ns", [40, 130])
+def test_image_outside_the_mask_is_cleared(ns, imaged):
+    """One segment (the gather clears) and three (the reduction does), with many
+    more runs outside the mask than warps, and with a few long ones."""
+    shape, dx, nt = (180, 200), 0.2e-3, 500
+    mask = np.zeros(shape, dtype=np.uint8)
+    if imaged == "few":
+        mask[85:95, 90:110] = 1
+    elif imaged == "scattered":
+        mask[::2, ::3] = 1
+    else:
+        mask[-1, -1] = 1
+    rng = np.random.default_rng(3)
+    sensors = np.zeros((ns, 3))
+    sensors[:, 1] = rng.uniform(0.0, 1.0, ns) * (shape[0] - 1) * dx
+    with BP.constant(1500.0, shape, dx, np.zeros(3), sensors, 1.2 * 0.054 / 1500.0 / nt, nt, mask=mask) as bp:
+        x = torch.randn(2, ns, nt, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+        out = torch.full(bp.out_shape(2), 7.0, device="cuda")
+        bp.reconstruct(x, out=out)
+        bp.sync()
+        outside = torch.from_numpy(mask == 0).cuda()
+        assert bool((out[:, outside] == 0).all()) and bool((out[:, ~outside] != 7.0).all())
+        for f in range(2):
+            one = bp.reconstruct(x[f:f + 1], out=torch.full(bp.out_shape(1), 7.0, device="cuda"))
+            assert torch.equal(one[0].view(torch.int32), out[f].view(torch.int32))
