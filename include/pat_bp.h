@@ -80,11 +80,12 @@ typedef void* pat_stream_t; /* a cudaStream_t; NULL = legacy default stream */
                                          gives the same bits                     */
 #define PAT_FLAG_NO_WINDOW 0x1000u /* unstaged single frames gather the
                                       integrand from L2 instead of from
-                                      shared-memory windows (the default
-                                      whenever every window has at most 384
-                                      samples; 288 with solid-angle weights;
-                                      constant speed: 192, and 128 pixels per
-                                      tile); same bits, for comparisons         */
+                                      shared-memory windows (the default where
+                                      every window has at most 384 samples, 288
+                                      with solid-angle weights, 128 at constant
+                                      speed and 192 with both, 128 pixels per
+                                      tile, and the launch fills its CTAs); same
+                                      bits, for comparisons                     */
 
 /* Read-only facts about a handle (pat_bp_info). */
 typedef struct {

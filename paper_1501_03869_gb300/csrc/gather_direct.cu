@@ -40,6 +40,7 @@
 
 #include "gather.cuh"
 #include "packed.cuh"
+#include "row_rules.h"
 
 namespace patbp {
 
@@ -364,7 +365,7 @@ __global__ void __launch_bounds__(256) direct_reduce_kernel(const __grid_constan
 constexpr int kWindowMaxRows = 384;  // largest slot (rows); longer windows take the kernel above
 
 template <int P, int SW, int FMT, int WB, int DELAYS, int WGT>
-__global__ void __launch_bounds__(128, DELAYS || WGT ? 6 : (WB > 288 ? 7 : 9))
+__global__ void __launch_bounds__(128, window_ctas(DELAYS, WGT, WB))
     gather_window_kernel(const __grid_constant__ DirectParams p) {
   constexpr int PW = P / 128;
   static_assert(PW * SW == 4, "a unit is four warps");
@@ -689,14 +690,9 @@ cudaError_t launch_gather_direct(const GatherConfig& c, int fmt, const InstDesc&
   dp.n_seg = d.n_seg;
   dp.G = d.G;
   dp.W = d.W;
-  // The windowed kernel when every window fits a slot.  Weights and computed
-  // delays hold more registers (6 CTAs per SM), and with computed delays the
-  // kernel above reads little besides the integrand: weights up to 288 rows
-  // (272 rows: 32.0 -> 30.7 us), computed delays up to 192 rows of 128-pixel
-  // tiles (120 rows: 549 -> 422 us; 360 rows 28.4 against 30.0, 256-pixel tiles
-  // 25.1 against 26.3).
-  const int most = c.delays ? (c.P == 128 ? 192 : 0) : (dp.wanchor ? 288 : kWindowMaxRows);
-  const bool window = !c.no_window && dp.W >= 0 && dp.W <= most && dp.G <= 64;
+  const bool window = !c.no_window && dp.G <= 64 &&
+                      window_pays(c.delays != 0, dp.wanchor != nullptr, c.P, dp.W,
+                                  int64_t(dp.n_tiles) * dp.n_seg, dp.n_seg, n_sm);
   if (window && c.P == 128 && c.SW == 4) return launch_window_mode<128, 4>(c.delays != 0, fmt, dp, n_sm, st, reduce);
   if (window && c.P == 256 && c.SW == 2) return launch_window_mode<256, 2>(c.delays != 0, fmt, dp, n_sm, st, reduce);
   if (c.P == 128 && c.SW == 4)

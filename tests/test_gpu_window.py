@@ -18,9 +18,9 @@ def _gpu():
         pytest.skip("no CUDA device")
 
 
-def _handle(mode, tile, ns, nt, extra):
+def _handle(mode, tile, ns, nt, extra, shape=(64, 70)):
     rng = np.random.default_rng(5)
-    shape, dx = (64, 70), 0.2e-3
+    dx = 0.2e-3
     speed = (1500.0 + 900.0 * synth.smooth_field(shape, 4.0, rng)).astype(np.float32)
     hi = (np.array(shape[::-1], dtype=float) - 1) * dx
     sensors = np.zeros((ns, 3))
@@ -84,3 +84,26 @@ def test_image_outside_the_mask_is_cleared(ns, imaged):
         for f in range(2):
             one = bp.reconstruct(x[f:f + 1], out=torch.full(bp.out_shape(1), 7.0, device="cuda"))
             assert torch.equal(one[0].view(torch.int32), out[f].view(torch.int32))
+
+
+@pytest.mark.parametrize("nt", [2000, 4500, 6000, 8500])
+@pytest.mark.parametrize("tile", [128, 256])
+@pytest.mark.parametrize("mode", ["table", "constant", "table_solid", "constant_solid"])
+def test_windowed_equals_unwindowed_in_full_waves(mode, tile, nt):
+    """Three segments of enough tiles that the windowed kernel takes every form
+    that has a slot (the smaller launches above leave some to the other kernel)."""
+    ns, shape = 130, (256, 256)
+    x = torch.randn(1, ns, nt, generator=torch.Generator("cuda").manual_seed(nt), device="cuda")
+    gpu = 0 if mode.startswith("constant") else _lib.PAT_FLAG_GPU_TABLE
+    with _handle(mode, tile, ns, nt, gpu, shape) as a, \
+            _handle(mode, tile, ns, nt, gpu | _lib.PAT_FLAG_NO_WINDOW, shape) as b:
+        assert a.info["n_tiles"] * a.info["split"] == (1536 if tile == 128 else 768)
+        sc = x.abs().amax(dim=2).contiguous()
+        for dtype in (torch.float32, torch.float16):
+            s = None if dtype == torch.float32 else sc
+            sig = x if s is None else (x / sc[..., None]).to(dtype).contiguous()
+            ia, ib = a.reconstruct(sig, scales=s), b.reconstruct(sig, scales=s)
+            assert torch.isfinite(ia).all() and bool((ia != 0).any())
+            assert torch.equal(ia.view(torch.int32), ib.view(torch.int32)), (dtype, a.info["window"])
+        a.sync()
+        b.sync()
