@@ -144,7 +144,7 @@ pat_status evict_locked(pat_bp_t h);
 pat_status reconstruct_locked(pat_bp_t h, const void* signals_dev, pat_dtype dtype,
                               const float* scales_dev, int n_frames, float* out_dev,
                               cudaStream_t stream, int* host_status = nullptr,
-                              bool* exported = nullptr);
+                              bool* exported = nullptr, bool over_link = false);
 pat_status restore_locked(pat_bp_t h, cudaStream_t st);
 // evict an idle handle by giving its device buffers to an evicted handle of the
 // same sizes (no synchronisation or allocation); false if the sizes differ

@@ -522,8 +522,9 @@ __device__ __forceinline__ void preprocess_group(const PreParams& p, int s, int 
 
 template <int DT, int FMT, int FB>
 __global__ void __launch_bounds__(256) preprocess_kernel(const PreParams p) {
-  // let the gather that depends on this kernel start its prologue now
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // let the gather that depends on this kernel start its prologue now (late: as
+  // the CTAs exit)
+  if (!p.late) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   preprocess_group<DT, FMT, FB>(p, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.z);
 }
 
@@ -579,8 +580,10 @@ size_t gather_smem_bytes(const GatherConfig& c, int Wst) {
 template <int DT, int FMT>
 static cudaError_t launch_pre_fb(const PreParams& p, cudaStream_t st) {
   dim3 grid(p.n_sensors, (p.n_frames + p.FB - 1) / p.FB);
-  // tiles: rows are split in time while that fills the chip (4 CTAs per SM)
-  if (p.FB >= 8) {
+  // tiles: rows are split in time while that fills the chip (4 CTAs per SM), but
+  // not 16-bit rows in host memory, of which every share would read all twice
+  // (16 BF16 frames of 128 sensors x 4 000 samples: 225 us in 2 shares, 125 whole)
+  if (p.FB >= 8 && !(DT != 0 && p.over_link)) {
     const int64_t chunks = (int64_t(p.n_t_pad) * p.FB + 4095) / 4096, rows = int64_t(grid.x) * grid.y;
     grid.z = unsigned(std::max<int64_t>(1, std::min<int64_t>(chunks, 4 * 152 / rows)));
   }

@@ -33,6 +33,8 @@ struct PreParams {
   float* m;              // [n_fg][N_s_pad][FB] multipliers w_s * sigma (0 for absent frames)
   int dtype, fmt, FB;
   int n_sensors, n_sensors_pad, n_t, n_t_pad, n_frames;
+  int late;              // 1: the gather may start once the last row is written, not from the start
+  int over_link;         // 1: the signals lie in host memory
 };
 
 // Preprocessing of several instances in one launch (same dtype, format, FB).

@@ -643,6 +643,7 @@ PreParams make_pre(pat_bp_t h, const void* sig, pat_dtype dtype, const float* sc
   pp.n_t = h->nt;
   pp.n_t_pad = h->nt_pad;
   pp.n_frames = n_frames;
+  pp.late = pp.over_link = 0;
   return pp;
 }
 
@@ -836,7 +837,8 @@ extern "C" pat_status pat_bp_reserve(pat_bp_t h, int max_frames, pat_dtype dtype
 }
 
 static pat_status preprocess_locked(pat_bp_t h, const void* signals_dev, pat_dtype dtype,
-                                    const float* scales_dev, int n_frames, cudaStream_t stream) {
+                                    const float* scales_dev, int n_frames, cudaStream_t stream,
+                                    bool over_link = false) {
   if (h->evicted) return fail(PAT_ERR_INVALID, "the handle's table is evicted (pat_bp_restore)");
   if (!signals_dev) return fail(PAT_ERR_INVALID, "signals NULL");
   if (n_frames < 1 || n_frames > 65535) return fail(PAT_ERR_INVALID, "n_frames must be 1..65535");
@@ -847,7 +849,17 @@ static pat_status preprocess_locked(pat_bp_t h, const void* signals_dev, pat_dty
   const int FB = pick_config(h, n_frames, fmt_for(dtype), &wst).FB;
   pat_status st = ensure_buffers_fb(h, n_frames, FB);
   if (st != PAT_OK) return st;
-  const PreParams pp = make_pre(h, signals_dev, dtype, scales_dev, n_frames, FB);
+  PreParams pp = make_pre(h, signals_dev, dtype, scales_dev, n_frames, FB);
+  // Signals read over the host link keep the preprocessing up for long, and its
+  // CTAs leave the SMs unevenly: a gather that starts in between puts all its
+  // CTAs for an SM, with a second unit each, on those that are free first.  Rows
+  // of 4, and of 8 with few units, lose most (4 frames of 21 300 pixels x 512
+  // sensors from host memory, 256-pixel tiles: 170 us, 150 when it starts with the
+  // last row; 5 frames, 128-pixel tiles 200, 195; 8 frames differ by 1 %).  From
+  // device memory the early start is worth 3 to 5 % to full launches.
+  const int64_t units = int64_t((n_frames + FB - 1) / FB) * h->n_tiles * h->n_seg;
+  pp.over_link = over_link;
+  pp.late = over_link && (FB == 4 || (FB == 8 && units < int64_t(6) * h->n_sm));
   cudaError_t e = launch_preprocess(pp, stream);
   if (e != cudaSuccess) return cuda_fail(e, "preprocess launch");
   h->pre_frames = n_frames;
@@ -910,10 +922,11 @@ static pat_status gather_locked(pat_bp_t h, int n_frames, float* out_dev, cudaSt
 
 pat_status patbp::reconstruct_locked(pat_bp_t h, const void* signals_dev, pat_dtype dtype,
                                       const float* scales_dev, int n_frames, float* out_dev,
-                                      cudaStream_t stream, int* host_status, bool* exported) {
+                                      cudaStream_t stream, int* host_status, bool* exported,
+                                      bool over_link) {
   if (!out_dev) return fail(PAT_ERR_INVALID, "out NULL");
   if (exported) *exported = false;
-  pat_status st = preprocess_locked(h, signals_dev, dtype, scales_dev, n_frames, stream);
+  pat_status st = preprocess_locked(h, signals_dev, dtype, scales_dev, n_frames, stream, over_link);
   if (st != PAT_OK) return st;
   return gather_locked(h, n_frames, out_dev, stream, host_status, exported);
 }
@@ -985,6 +998,7 @@ extern "C" pat_status pat_bp_reconstruct_host(pat_bp_t h, const void* signals_ho
   // in place and the last kernel writes the image in place -- no staging
   // copies.  Pageable buffers go through device staging buffers.
   const void* sig_dev = device_address(signals_host);
+  const bool over_link = sig_dev != nullptr;
   const float* sc_dev = scales_host ? static_cast<const float*>(device_address(scales_host)) : nullptr;
   float* out_dev = static_cast<float*>(device_address(out_host));
   if (!sig_dev) {
@@ -1013,7 +1027,7 @@ extern "C" pat_status pat_bp_reconstruct_host(pat_bp_t h, const void* signals_ho
   }
   *reinterpret_cast<volatile int*>(h->host_status) = 0;
   bool exported = false;
-  st = reconstruct_locked(h, sig_dev, dtype, sc_dev, n_frames, out_dev, s, h->host_status_dev, &exported);
+  st = reconstruct_locked(h, sig_dev, dtype, sc_dev, n_frames, out_dev, s, h->host_status_dev, &exported, over_link);
   if (st != PAT_OK) return st;
   if (out_staged) PAT_CUDA(cudaMemcpyAsync(out_host, out_dev, out_bytes, cudaMemcpyDeviceToHost, s));
   if (!exported) PAT_CUDA(launch_status_export(h->d_status, h->host_status_dev, s));

@@ -128,3 +128,20 @@ def test_reserved_handle_allocates_nothing_for_shorter_rows(reserved, frames):
         assert torch.equal(out.view(torch.int32), want.view(torch.int32))
         bp.sync()
         ref.sync()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("tile", [128, 256])
+def test_page_locked_signals(tile, dtype):
+    """Signals read over the host link, for which rows of 4 hold the gather's
+    start back: the bits of device signals, call after call."""
+    with _handle((72, 80), 150, 301, tile, "table") as bp:
+        for n in (4, 6, 8, 12, 4):
+            sig, sc = _signals(n, 150, 301, dtype, n)
+            want = bp.reconstruct(sig, scales=sc).cpu()
+            bp.sync()
+            host = (sig if sc is None else sig.view(torch.int16)).cpu().pin_memory().numpy()
+            out = torch.full_like(want, 7.0).pin_memory()
+            bp.reconstruct_host(host if sc is None else host.view(np.uint16), dtype=dtype,
+                                scales=None if sc is None else sc.cpu().pin_memory().numpy(), out=out.numpy())
+            assert torch.equal(out.view(torch.int32), want.view(torch.int32))
