@@ -695,42 +695,64 @@ __global__ void __launch_bounds__(RowsShape<P, FB, FMT, MODE>::THREADS, RowsShap
 // Sum of the segment sums of a split launch, in segment order, written to the
 // image.  FB / 4 neighbouring lanes take the frames of one pixel (16 bytes
 // each): whole rows of the partial sums are read; 8 segments are in flight.
+// Lanes of rows of 16 and 32 frames hold few neighbouring pixels of a frame; their
+// sums are turned in shared memory, so that a warp writes 32 (into an image in host
+// memory, pieces of 4 pixels took 122 us for 32 frames of 21 300; small launches
+// with short rows would only lose a microsecond).
 template <int FB>
 __global__ void __launch_bounds__(256) rows_reduce_kernel(const __grid_constant__ StreamParams p, int P) {
   constexpr int LPP = FB / 4, K = 8;
+  constexpr bool TURN = FB >= 16;
+  constexpr int PX = 256 / LPP, PITCH = PX + 8 / LPP;  // pixels of one pass; no bank twice
+  __shared__ float turned[TURN ? FB : 1][TURN ? PITCH : 1];
   asm volatile("griddepcontrol.wait;" ::: "memory");
   for (int i = 0; i < p.n_inst; ++i) {
     const InstDesc& d = p.inst[i];
     if (d.n_seg == 1) continue;  // written by the gather
-    const int64_t n = int64_t(d.n_fg) * d.n_tiles * P * LPP;
-    for (int64_t idx = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; idx < n;
-         idx += int64_t(gridDim.x) * blockDim.x) {
-      const int lq = int(idx % LPP);
-      const int64_t pxl = idx / LPP;
-      const int64_t ft = pxl / P;  // frame group * n_tiles + tile
-      const int px = int(pxl - ft * P);
-      const int fg = int(ft / d.n_tiles), tile = int(ft - int64_t(fg) * d.n_tiles);
-      const int o = __ldcg(d.slot + int64_t(tile) * P + px);
-      const float4* src = reinterpret_cast<const float4*>(d.part + (ft * d.n_seg * P + px) * FB) + lq;
-      const int64_t step = int64_t(P) * LPP;
+    const int64_t n = int64_t(d.n_fg) * d.n_tiles * P;  // pixels of all frame groups
+    for (int64_t first = int64_t(blockIdx.x) * PX; first < n; first += int64_t(gridDim.x) * PX) {
+      // what this thread adds: a quad of frames of a pixel; what it writes: that,
+      // or the frames f0, f0 + LPP, .. of another
+      const int lq = int(threadIdx.x) % LPP, mine = int(threadIdx.x) / LPP;
+      const int at = TURN ? int(threadIdx.x) % PX : mine, f0 = TURN ? int(threadIdx.x) / PX : lq * 4;
+      int o = -1, fg = 0;
+      if (first + at < n) {
+        fg = int((first + at) / P / d.n_tiles);
+        o = __ldcg(d.slot + first + at - int64_t(fg) * d.n_tiles * P);
+      }
       float4 t = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      for (int s0 = 0; s0 < d.n_seg; s0 += K) {
-        float4 x[K];
+      if (first + mine < n) {
+        const int64_t ft = (first + mine) / P;  // frame group * n_tiles + tile
+        const int px = int(first + mine - ft * P);
+        const float4* src = reinterpret_cast<const float4*>(d.part + (ft * d.n_seg * P + px) * FB) + lq;
+        const int64_t step = int64_t(P) * LPP;
+        for (int s0 = 0; s0 < d.n_seg; s0 += K) {
+          float4 x[K];
 #pragma unroll
-        for (int k = 0; k < K; ++k)
-          x[k] = s0 + k < d.n_seg ? __ldcg(src + (s0 + k) * step) : make_float4(0.f, 0.f, 0.f, 0.f);
+          for (int k = 0; k < K; ++k)
+            x[k] = s0 + k < d.n_seg ? __ldcg(src + (s0 + k) * step) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-          if (s0 + k >= d.n_seg) break;
-          t.x += x[k].x; t.y += x[k].y; t.z += x[k].z; t.w += x[k].w;
+          for (int k = 0; k < K; ++k) {
+            if (s0 + k >= d.n_seg) break;
+            t.x += x[k].x; t.y += x[k].y; t.z += x[k].z; t.w += x[k].w;
+          }
         }
       }
-      if (o < 0) continue;
-      const float v[4] = {t.x, t.y, t.z, t.w};
-      const int f0 = fg * FB + lq * 4;
+      float v[4] = {t.x, t.y, t.z, t.w};
+      if constexpr (TURN) {
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
-        if (f0 + k < d.n_frames) d.out[int64_t(f0 + k) * d.out_stride + o] = v[k];
+        for (int k = 0; k < 4; ++k) turned[lq * 4 + k][mine] = v[k];
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = turned[f0 + k * LPP][at];
+        __syncthreads();
+      }
+      if (o < 0) continue;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int f = fg * FB + f0 + (TURN ? k * LPP : k);
+        if (f < d.n_frames) d.out[int64_t(f) * d.out_stride + o] = v[k];
+      }
     }
   }
 }
