@@ -582,10 +582,11 @@ static cudaError_t launch_pre_fb(const PreParams& p, cudaStream_t st) {
   dim3 grid(p.n_sensors, (p.n_frames + p.FB - 1) / p.FB);
   // tiles: rows are split in time while that fills the chip (4 CTAs per SM), but
   // not 16-bit rows in host memory, of which every share would read all twice
-  // (16 BF16 frames of 128 sensors x 4 000 samples: 225 us in 2 shares, 125 whole)
+  // (16 BF16 frames of 128 sensors x 4 000 samples: 225 us in 2 shares, 125 whole);
+  // FP32 rows there in half as many (32 frames of 64 sensors: 48 us in 2, 44 whole)
   if (p.FB >= 8 && !(DT != 0 && p.over_link)) {
     const int64_t chunks = (int64_t(p.n_t_pad) * p.FB + 4095) / 4096, rows = int64_t(grid.x) * grid.y;
-    grid.z = unsigned(std::max<int64_t>(1, std::min<int64_t>(chunks, 4 * 152 / rows)));
+    grid.z = unsigned(std::max<int64_t>(1, std::min<int64_t>(chunks, int64_t(p.over_link ? 2 : 4) * p.n_sm / rows)));
   }
   switch (p.FB) {
     case 1: preprocess_kernel<DT, FMT, 1><<<grid, 256, 0, st>>>(p); break;

@@ -35,6 +35,7 @@ struct PreParams {
   int n_sensors, n_sensors_pad, n_t, n_t_pad, n_frames;
   int late;              // 1: the gather may start once the last row is written, not from the start
   int over_link;         // 1: the signals lie in host memory
+  int n_sm;              // multiprocessors of the device
 };
 
 // Preprocessing of several instances in one launch (same dtype, format, FB).

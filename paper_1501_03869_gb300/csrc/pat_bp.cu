@@ -644,6 +644,7 @@ PreParams make_pre(pat_bp_t h, const void* sig, pat_dtype dtype, const float* sc
   pp.n_t_pad = h->nt_pad;
   pp.n_frames = n_frames;
   pp.late = pp.over_link = 0;
+  pp.n_sm = h->n_sm;
   return pp;
 }
 
