@@ -847,7 +847,15 @@ static pat_status preprocess_locked(pat_bp_t h, const void* signals_dev, pat_dty
     return fail(PAT_ERR_INVALID, "unknown dtype");
   if (dtype != PAT_F32 && !scales_dev) return fail(PAT_ERR_INVALID, "16-bit signals need scales");
   int wst = 0;
-  const int FB = pick_config(h, n_frames, fmt_for(dtype), &wst).FB;
+  int FB = pick_config(h, n_frames, fmt_for(dtype), &wst).FB;
+  int64_t units = int64_t((n_frames + FB - 1) / FB) * h->n_tiles * h->n_seg;
+  // Host to host, one segment, few units: the gather writes the image itself, and
+  // rows of 4 write neighbouring pixels where rows of 8 leave gaps of a frame
+  // each (32 FP32 frames of 64 sensors x 6 092 pixels: 103 us in rows of 8, 84 of 4)
+  if (over_link && h->n_seg == 1 && FB == 8 && units < int64_t(6) * h->n_sm) {
+    FB = pick_config(h, n_frames, fmt_for(dtype), &wst, 4).FB;
+    units = int64_t((n_frames + FB - 1) / FB) * h->n_tiles * h->n_seg;
+  }
   pat_status st = ensure_buffers_fb(h, n_frames, FB);
   if (st != PAT_OK) return st;
   PreParams pp = make_pre(h, signals_dev, dtype, scales_dev, n_frames, FB);
@@ -858,7 +866,6 @@ static pat_status preprocess_locked(pat_bp_t h, const void* signals_dev, pat_dty
   // sensors from host memory, 256-pixel tiles: 170 us, 150 when it starts with the
   // last row; 5 frames, 128-pixel tiles 200, 195; 8 frames differ by 1 %).  From
   // device memory the early start is worth 3 to 5 % to full launches.
-  const int64_t units = int64_t((n_frames + FB - 1) / FB) * h->n_tiles * h->n_seg;
   pp.over_link = over_link;
   pp.late = over_link && (FB == 4 || (FB == 8 && units < int64_t(6) * h->n_sm));
   cudaError_t e = launch_preprocess(pp, stream);
