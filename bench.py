@@ -159,12 +159,13 @@ def kernel_source_hash():
 
 def single_frame_kernels(info):
     """Names of the two kernels one FP32 frame of a stored table takes: the
-    windowed gather when every window fits its largest slot (384 rows)."""
+    windowed gather up to 288 rows per window (above, up to 384, only where the
+    launch fills its CTAs; the workloads here have shorter windows)."""
     P = info["tile_pix"]
     sw = 4 if P == 128 else 2
     W = info["window"]
-    if W <= 384:
-        wb = next(b for b in (128, 192, 288, 384) if W <= b)
+    if W <= 288:
+        wb = next(b for b in (128, 192, 288) if W <= b)
         return f"gather_window_kernel<{P},{sw},f32,{wb}> + direct_reduce_kernel<{P},1>"
     return f"gather_direct_kernel<{P},{sw},f32,table> + direct_reduce_kernel<{P},{sw}>"
 

@@ -1,11 +1,11 @@
 // gather_direct.cu -- the single-frame gather of Eq. (BP) without the staged
 // pipeline.
 //
-// Two gathers share the reduction kernel below.  gather_window_kernel (every
-// window at most 384 samples) copies each sensor's integrand window into
-// shared memory per warp and interpolates there; gather_direct_kernel,
-// described next, gathers from L2 and takes every other case.  Both give the
-// same bits.
+// Two gathers share the reduction kernel below.  gather_window_kernel (windows
+// that fit a slot, and launches that fill its CTAs: window_pays in row_rules.h)
+// copies each sensor's integrand window into shared memory per warp and
+// interpolates there; gather_direct_kernel, described next, gathers from L2 and
+// takes every other case.  Both give the same bits.
 //
 // Two launches.  The gather kernel is persistent: CTA c takes units (tile,
 // segment of G sensors) c, c + grid, c + 2 grid, ... in tile-major order, and
@@ -186,24 +186,18 @@ __global__ void __launch_bounds__(32 * (P / 128) * SW, kDirectMinCtas)
       for (int c0 = s_lo + sp; c0 < s_hi; c0 += CH * SW) {
         uint32_t bw[CH];
         float uu[CH][4];
-        float4 an[DELAYS ? CH : 1][2];
+        float4 an[CH][2];
         float4 wa[WGT ? CH : 1][2];
   #pragma unroll
         for (int j = 0; j < CH; ++j) {
           const int s = c0 + j * SW;
           const bool ok = s < s_hi;
           bw[j] = ok ? uint32_t(__ldcg(p.base + int64_t(tile) * p.n_sensors_pad + s)) : 0u;
-          if constexpr (DELAYS == 0) {
-            const float* urow = p.u + (int64_t(tile) * p.n_sensors + s) * P + px0;
-  #pragma unroll
-            for (int x = 0; x < 4; ++x) uu[j][x] = ok ? __ldcg(urow + x * 32) : kFarOffset;
-          } else {
-            const float4* ap = reinterpret_cast<const float4*>(p.anchor) +
-                               (int64_t(tile) * p.n_sensors_pad + (ok ? s : s_lo)) * 2;
-            an[j][0] = __ldcg(ap);
-            an[j][1] = __ldcg(ap + 1);
-            if (!ok) an[j][1].y = -1.0f;  // cap below every offset: nothing to add
-          }
+          const float4* ap = reinterpret_cast<const float4*>(p.anchor) +
+                             (int64_t(tile) * p.n_sensors_pad + (ok ? s : s_lo)) * 2;
+          an[j][0] = __ldcg(ap);
+          an[j][1] = __ldcg(ap + 1);
+          if (!ok) an[j][1].y = -1.0f;  // cap below every offset: nothing to add
           if constexpr (WGT != 0) {
             wa[j][0] = __ldcg(wrow + 2 * (ok ? s : s_lo));
             wa[j][1] = __ldcg(wrow + 2 * (ok ? s : s_lo) + 1);
@@ -220,30 +214,28 @@ __global__ void __launch_bounds__(32 * (P / 128) * SW, kDirectMinCtas)
   #pragma unroll
         for (int j = 0; j < CH; ++j) {
           const int s = min(c0 + j * SW, s_hi - 1);
-          if constexpr (DELAYS != 0) {
-            const float4 A = an[j][0], B = an[j][1];
-            if (B.w == 0.0f) {
-              const float m2u0 = -2.0f * A.w;
+          const float4 A = an[j][0], B = an[j][1];
+          if (B.w == 0.0f) {
+            const float m2u0 = -2.0f * A.w;
   #pragma unroll
-              for (int x = 0; x < 4; ++x) {
-                const float num =
-                    fmaf(pq[x].x, A.x, fmaf(pq[x].y, A.y, fmaf(pq[x].z, A.z, pq[x].w)));
-                const float sq = num + B.z;
-                const float y = rsqrtf(sq);
-                const float da = sq * y - A.w;
-                const float r = fmaf(-da, da, fmaf(m2u0, da, num));
-                const float v = fmaf(r, 0.5f * y, da) + B.x;
-                uu[j][x] = v > B.y ? kFarOffset : fmaxf(v, 0.0f);
-              }
-            } else {
+            for (int x = 0; x < 4; ++x) {
+              const float num =
+                  fmaf(pq[x].x, A.x, fmaf(pq[x].y, A.y, fmaf(pq[x].z, A.z, pq[x].w)));
+              const float sq = num + B.z;
+              const float y = rsqrtf(sq);
+              const float da = sq * y - A.w;
+              const float r = fmaf(-da, da, fmaf(m2u0, da, num));
+              const float v = fmaf(r, 0.5f * y, da) + B.x;
+              uu[j][x] = v > B.y ? kFarOffset : fmaxf(v, 0.0f);
+            }
+          } else {
   #pragma unroll
-              for (int x = 0; x < 4; ++x) {
-                const float d0 = fmaf(0.5f, pq[x].x, A.x), d1 = fmaf(0.5f, pq[x].y, A.y),
-                            d2 = fmaf(0.5f, pq[x].z, A.z);
-                const float sq = fmaxf(fmaf(d0, d0, fmaf(d1, d1, d2 * d2)), 1.0e-30f);
-                const float v = (sq * rsqrtf(sq) - A.w) + B.x;
-                uu[j][x] = v > B.y ? kFarOffset : fmaxf(v, 0.0f);
-              }
+            for (int x = 0; x < 4; ++x) {
+              const float d0 = fmaf(0.5f, pq[x].x, A.x), d1 = fmaf(0.5f, pq[x].y, A.y),
+                          d2 = fmaf(0.5f, pq[x].z, A.z);
+              const float sq = fmaxf(fmaf(d0, d0, fmaf(d1, d1, d2 * d2)), 1.0e-30f);
+              const float v = (sq * rsqrtf(sq) - A.w) + B.x;
+              uu[j][x] = v > B.y ? kFarOffset : fmaxf(v, 0.0f);
             }
           }
           const unsigned bs = bw[j] & 0xffffu;
