@@ -62,11 +62,12 @@ struct RowsShape {
   static constexpr int V = A < 4 ? A : (NQ == 2 ? 4 : 2); // of which neighbours in the tile
   static constexpr int THREADS = 32 * (NW + 1 + NC);
   // resident CTAs per SM the registers must allow: 11 to 18 warps.  8-frame rows
-  // spill in the 96 registers of three where a lane owns four pixels (256-pixel
-  // tiles) or computes offsets or weights: two are faster there (24 FP32 frames
-  // as above, 256-pixel tiles 184 -> 166 us; 12 frames of 6 600 pixels x 128
-  // sensors, constant speed 34 -> 28 us, with weights too 39 -> 31).
-  static constexpr int MIN_CTAS = FB >= 16 ? 1 : (FB == 8 && (P == 256 || MODE != 0) ? 2 : 3);
+  // spill in the 96 registers of three where a lane computes offsets or weights:
+  // two are faster there (24 FP32 frames as above, constant speed, 256-pixel tiles
+  // 234 -> 204 us; 12 frames of 6 600 pixels x 128 sensors 34 -> 28 us, with weights
+  // too 39 -> 31).  With a table one call of 24 frames gains as well (184 -> 166),
+  // but 32 uneven instances lose (2.62 -> 2.81 ms).
+  static constexpr int MIN_CTAS = FB >= 16 ? 1 : (FB == 8 && MODE != 0 ? 2 : 3);
   static_assert(A % V == 0 && NPX * NW == P, "pixels of a lane");
 };
 

@@ -562,16 +562,14 @@ void ring_need(GatherConfig c, int longest, size_t* fixed, size_t* window) {
 // SM (one CTA of 8 consumer warps; half the ring is 1.2 to 1.8 times slower),
 // 8-frame rows three CTAs of 4 consumer warps (8 frames of 1.04 M voxels,
 // BF16: 2.12 ms; two CTAs 2.60, four 2.41) or the two that their registers allow
-// (24 FP32 frames of 22 300 pixels x 512 sensors, 256-pixel tiles: 166 us in 110
-// KB, 184 in 72), groups of 8 sensors where 128-pixel tiles compute offsets or
-// weights (8 frames of 0.3 M voxels x 256 sensors, weights: 351 us, 458 in groups
-// of 4).
+// with computed delays or weights, there in groups of 8 sensors for 128-pixel tiles
+// (8 frames of 0.3 M voxels x 256 sensors, weights: 351 us, 458 in groups of 4).
 void default_shape(const GatherConfig& c, size_t limit, int* S, size_t* budget) {
   static const int s[6] = {16, 8, 8, 4, 8, 4}, kb[6] = {72, 100, 72, 72, 0, 0};
   const int i = fb_index(c.FB);
   const bool mode = c.delays || c.wgt;
   *S = c.FB == 8 && c.P == 128 && mode ? 8 : s[i];
-  *budget = kb[i] ? size_t(c.FB == 8 && (c.P == 256 || mode) ? 110 : kb[i]) * 1024 : limit;
+  *budget = kb[i] ? size_t(c.FB == 8 && mode ? 110 : kb[i]) * 1024 : limit;
 }
 
 // Launch shape for a frame count: the autotuned one when the handle has it,

@@ -4,7 +4,7 @@
 // work to a persistent gather launch.  Instances are grouped by the frames
 // that share one pass over a table tile (FB: the largest power of two up to
 // 8 not above the instance's frame count; 16 or 32 above 16 frames where that
-// pads no further), and every group ("class") has its own preprocessing launch
+// pads no further and choose_frames_per_unit finds it faster), and every group ("class") has its own preprocessing launch
 // (the Eq. (BP) integrand of all its instances), its own gather launch and,
 // from 4 frames per unit on, the launch that adds its segments; all
 // preprocessing launches go first, then the gathers.  A 16-frame instance
@@ -113,6 +113,17 @@ int class_window(pat_plan_t pl, const std::vector<int>& idx, int S) {
   return w;
 }
 
+// Mean over a class's units of their instances' longest windows.
+int class_mean_window(pat_plan_t pl, const std::vector<int>& idx, int FB) {
+  int64_t units = 0, rows = 0;
+  for (int i : idx) {
+    const int64_t u = int64_t((pl->frames[i] + FB - 1) / FB) * pl->hs[i]->n_tiles * pl->hs[i]->n_seg;
+    units += u;
+    rows += u * stage_window(pl->hs[i], 1);
+  }
+  return units > 0 ? int(rows / units) : 8;
+}
+
 // Frames per unit of every instance.  Rows of 32 or 16 frames are halved, down
 // to 8, for a class whose units (frame group, tile, segment) would not fill the
 // chip -- fewer than four per SM in rows of 32, one in rows of 16 -- and for an
@@ -169,7 +180,7 @@ pat_status plan_shape(pat_plan_t pl, int S, int budget_kb) {
       default_shape(c, limit, &Sk, &budget);
       if (k.FB >= 4) {
         size_t fixed = 0, window = 0;
-        ring_need(c, wmin, &fixed, &window);
+        ring_need(c, class_mean_window(pl, k.idx, k.FB), &fixed, &window);
         budget = ring_budget(budget, fixed, window, k.FB, limit);
       }
       pl->S = std::max(pl->S, Sk);

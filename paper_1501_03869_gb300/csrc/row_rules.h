@@ -22,16 +22,19 @@ inline bool ring_is_deep(int FB, size_t fixed, size_t window, size_t limit) {
   return fixed + (FB == 4 ? 4 : 3) * window <= limit;
 }
 
-// Shared-memory budget where `budget` is the one for short windows: the
-// smallest of it, 110 KB and the device's limit whose ring holds 32 / FB of the
-// longest windows.  8 FP32 frames of 22 300 pixels x 512 sensors with windows of
-// 320 / 632 rows: 87 / 130 us in 72 KB, 89 / 117 in 110 KB, 120 / 133 in all; 4
-// frames with 632 / 1 248 rows: 79 / 120 us, 74 / 113, 81 / 112.
+// Shared-memory budget where `budget` is the one for short windows: that while its
+// ring holds 32 / FB of the longest windows, else 110 KB while that holds two and a
+// half, else the device's limit.  8 FP32 frames of 22 300 pixels x 512 sensors with
+// windows of 320 / 632 / 1 248 rows: 87 / 130 us in 72 KB, 89 / 117 / 184 in 110
+// KB, 120 / 133 / 184 in all; 4 frames with 632 / 1 248 rows: 79 / 120 us, 74 / 113,
+// 81 / 112.  (For a class of a plan, `window` is the mean over its instances' units:
+// one long record must not leave 32 uneven instances a CTA per SM, 3.80 ms against
+// 2.67.)
 inline size_t ring_budget(size_t budget, size_t fixed, size_t window, int FB, size_t limit) {
-  const size_t need = fixed + size_t(32 / FB) * window;
-  if (need <= budget) return budget;
   const size_t two = size_t(110) * 1024;
-  return budget < two && two <= limit && need <= two ? two : limit;
+  if (fixed + size_t(32 / FB) * window <= budget) return budget;
+  if (budget < two && two <= limit) budget = two;
+  return fixed + window * 5 / 2 <= budget ? budget : limit;
 }
 
 // Resident CTAs per SM of the windowed single-frame gather: what its registers

@@ -26,7 +26,7 @@ int main() {
       // the default until the ring gets shallow, and never more than needed
       if (fixed + 32 / FB * window <= first) need(b == first, "short windows leave the default", FB, rows);
       else need(b > first || first == limit, "long windows in the default budget", FB, rows);
-      if (b < limit) need(fixed + 32 / FB * window <= b, "a shallow ring below the limit", FB, rows);
+      if (b < limit) need(fixed + 5 * window / 2 <= b, "a shallow ring below the limit", FB, rows);
       // rows whose ring holds fewer than three windows give way (rows of 4: four)
       need(ring_is_deep(FB, fixed, window, limit) == ((limit - fixed) / window >= (FB == 4 ? 4u : 3u)), "deep", FB, rows);
     }
@@ -34,7 +34,9 @@ int main() {
   // what rows of 32 cannot hold, rows of 8 can
   need(!ring_is_deep(32, fixed, 1752 * 128, limit) && ring_is_deep(8, fixed, 1752 * 32, limit), "1 752 rows", 32, 1752);
   need(ring_budget(72 * 1024, fixed, 12000, 8, 100 * 1024) == 72 * 1024, "a device with less", 8, 0);
-  need(ring_budget(72 * 1024, fixed, 22000, 8, 100 * 1024) == 100 * 1024, "a device with less than 110 KB", 8, 0);
+  need(ring_budget(72 * 1024, fixed, 40000, 8, 100 * 1024) == 100 * 1024, "a device with less than 110 KB", 8, 0);
+  need(ring_budget(110 * 1024, fixed, 30000, 8, limit) == 110 * 1024 && ring_budget(110 * 1024, fixed, 45000, 8, limit) == limit,
+       "from 110 KB", 8, 0);
   const int n_sm = 152;
   auto pays = [&](bool delays, bool weights, int P, int rows, int64_t units, int n_seg) {
     return window_pays(delays, weights, P, rows, units, n_seg, n_sm);

@@ -180,9 +180,9 @@ def test_noalloc_at_the_scratch_limit():
             bp.reconstruct_noalloc(more, torch.empty(bp.out_shape(33), device="cuda"))
 
 
-@pytest.mark.parametrize("frames,nt,budget", [(8, 2001, 72), (8, 6001, 110), (8, 9001, 200), (5, 6001, 110)])
+@pytest.mark.parametrize("frames,nt,budget", [(8, 2001, 72), (8, 6001, 110), (8, 14000, 200), (5, 6001, 110)])
 def test_plans_widen_the_ring_for_long_windows(frames, nt, budget):
-    """Windows of 240, 712 and 1 072 rows of 8 frames, 712 of 4: the budget
+    """Windows of 240, 728 and 1 672 rows of 8 frames, 728 of 4: the budget
     grows before a ring gets down to one group."""
     with _handle((72, 80), 12, nt) as bp:
         info = _check_plan([bp], [frames])
@@ -220,13 +220,13 @@ def test_reserved_handle_allocates_nothing_for_long_windows(frames, nt):
 def test_shapes_of_computed_delays(tile, dtype):
     """Constant speed: 16-bit frames take rows of 8 where FP32 takes 16, and
     8-frame rows get the shared memory of two CTAs per SM, whose registers hold
-    what three would spill; stored delays of 128-pixel tiles keep three."""
+    what three would spill; stored delays keep three."""
     with _handle((160, 160), 256, 401, tile, "constant") as bp, _handle((160, 160), 256, 401, tile) as table:
         assert _check_plan([bp], [48], dtype)["fb_mask"] == (16 if dtype == "f32" else 8)
         info = _check_plan([bp], [8], dtype)
         assert info["smem_budget_kb"] == 110 and info["sensors_per_stage"] == (8 if tile == 128 else 4)
         info = _check_plan([table], [8], dtype)
-        assert info["smem_budget_kb"] == (72 if tile == 128 else 110)
+        assert info["smem_budget_kb"] == 72
         _set_weights(bp, 256)
         assert _check_plan([bp], [48], dtype)["fb_mask"] == (16 if dtype == "f32" else 8)
         assert _check_plan([bp], [24], dtype)["smem_budget_kb"] == 110
