@@ -358,18 +358,25 @@ __global__ void __launch_bounds__(RowsShape<P, FB, FMT, MODE>::THREADS, RowsShap
           sg.stride = uint64_t(d.n_t_pad) * ROW;
         }
         __syncwarp();
-        // lane k: rows of the segment's sensors before (k + 1) S
-        const int last = min(n, (lane + 1) * p.S) - 1;
-        const uint32_t u0 = __shfl_sync(0xffffffffu, a0, last & 31), u1 = __shfl_sync(0xffffffffu, a1, last & 31);
-        const uint32_t upto = last < 32 ? u0 : u1;
+        // Groups of up to S sensors as their windows come, each at most a third of
+        // the ring: one long window in a class must not cut every group down to the
+        // two sensors that would fit with it.  They end on whole turns of the phases
+        // where there are as many.
         uint32_t before = 0;
-        for (int i0 = 0, k = 0; i0 < n && ok; i0 += p.S, ++k) {
-          const uint32_t to = __shfl_sync(0xffffffffu, upto, k & 31);
-          // (up to 64 groups of one sensor: the second 32 need their own counts)
-          uint32_t t2 = to;
-          if (k >= 32) t2 = __shfl_sync(0xffffffffu, a1, k & 31);
-          ok = publish(min(p.S, n - i0), i0, sgi, t2 - before);
-          before = t2;
+        for (int i0 = 0; i0 < n && ok;) {
+          const int at = i0 + lane;
+          const uint32_t u0 = __shfl_sync(0xffffffffu, a0, at & 31), u1 = __shfl_sync(0xffffffffu, a1, at & 31);
+          const uint32_t upto = at < 32 ? u0 : u1;  // rows up to this sensor
+          const bool in = lane < p.S && at < n &&
+                          RowsGroup(lane + 1, P, FB, MODE).bytes(int(upto - before), FB) <= ring_bytes / kRowsShare;
+          int se = max(1, __popc(__ballot_sync(0xffffffffu, in)));
+          const int turn = i0 & (SW - 1);
+          if (turn) se = min(se, SW - turn);
+          else if (se > SW) se &= ~(SW - 1);
+          const uint32_t to = __shfl_sync(0xffffffffu, upto, se - 1);
+          ok = publish(se, i0, sgi, to - before);
+          before = to;
+          i0 += se;
         }
         if (++sgi == kSegs) sgi = 0;
       }

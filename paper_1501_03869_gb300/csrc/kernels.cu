@@ -649,7 +649,7 @@ static cudaError_t rows_dispatch(const GatherConfig& c, int fmt, const StreamPar
 }
 
 size_t rows_group_bytes(const GatherConfig& c, int rows) {
-  return RowsGroup(c.S, c.P, c.FB, c.delays | (c.wgt << 1)).bytes(rows, c.FB);
+  return RowsGroup(1, c.P, c.FB, c.delays | (c.wgt << 1)).bytes(rows, c.FB);
 }
 
 const void* rows_reduce_func(int FB) {
@@ -742,7 +742,7 @@ cudaError_t launch_gather(const GatherConfig& c, int fmt, const StreamParams& p,
     return cudaSuccess;
   }
   if (c.FB >= 4) {
-    // any group of the launch must fit the ring
+    // any sensor of the launch must fit the ring
     if (p.ring != c.ring || p.ring % 128 || p.S > kRowsMaxS || rows_group_bytes(c, p.Wst) > size_t(p.ring)) return cudaErrorInvalidValue;
     return launch_rows(c, fmt, p, grid, st);
   }

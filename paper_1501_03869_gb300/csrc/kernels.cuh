@@ -101,7 +101,7 @@ struct GatherConfig {
 };
 
 size_t gather_smem_bytes(const GatherConfig& c, int Wst);
-// Ring bytes of a batched gather's group of S sensors with `rows` window rows.
+// Ring bytes of one sensor of a batched gather with `rows` window rows.
 size_t rows_group_bytes(const GatherConfig& c, int rows);
 // CTAs of one gather launch that fit on the device at once.
 int gather_resident_ctas(const GatherConfig& c, int fmt, int Wst, int n_sm);

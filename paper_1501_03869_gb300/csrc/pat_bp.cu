@@ -493,13 +493,12 @@ int stage_window(pat_bp_t h, int S) {
 // two stages with whatever fits above wmin.  False if even that does not fit.
 bool fit_stages(GatherConfig& c, int wmin, int wfull, size_t budget, int* wst) {
   if (c.FB >= 4) {
-    // the whole budget is one ring; any group of S sensors must fit it (wfull
-    // rows, the longest sum over the S-sensor groups)
+    // the whole budget is one ring, and any sensor must fit it
     c.stages = 1;
     c.ring = 0;
-    const size_t fixed = gather_smem_bytes(c, 0), need = rows_group_bytes(c, wfull);
+    const size_t fixed = gather_smem_bytes(c, 0), need = rows_group_bytes(c, wmin);
     c.ring = int(budget > fixed ? (budget - fixed) & ~size_t(127) : 0);
-    *wst = wfull;
+    *wst = wmin;
     if (c.ring >= int(need)) return true;
     c.ring = int(need);
     return false;
@@ -539,11 +538,7 @@ GatherConfig config_for(pat_bp_t h, int n_frames, int FB, int S, size_t budget, 
     const bool ok = fit_stages(c, wmin, stage_window(h, c.S), budget, wst);
     if (fits) *fits = ok;
     if (ok) break;
-    if (FB >= 4 && c.S > 1) {
-      c.S /= 2;
-      continue;
-    }
-    if (c.S <= 4) break;
+    if (FB >= 4 || c.S <= 4) break;
     c.S /= 2;
   }
   return c;

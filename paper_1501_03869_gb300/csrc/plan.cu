@@ -193,14 +193,8 @@ pat_status plan_shape(pat_plan_t pl, int S, int budget_kb) {
     c.S = Sk;
     int wst = wfull;
     bool fits = fit_stages(c, wmin, wfull, budget, &wst);
-    if (k.FB >= 4)  // smaller groups of sensors where the longest sums do not fit
-      while (!fits && c.S > 1) {
-        c.S /= 2;
-        wfull = class_window(pl, k.idx, c.S);
-        fits = fit_stages(c, wmin, wfull, budget, &wst);
-      }
     if (!fits && S == 0 && budget < limit) {  // a default shape too small for long windows: the whole SM
-      c.S = 4;
+      if (k.FB < 4) c.S = 4;
       wfull = class_window(pl, k.idx, c.S);
       fits = fit_stages(c, wmin, wfull, limit, &wst);
     }

@@ -30,6 +30,7 @@ namespace patbp {
 
 constexpr int kSlots = 8;
 constexpr int kRowsMaxS = 16;  // sensors of a group
+constexpr int kRowsShare = 3;  // a group of several sensors takes at most this part of the ring
 constexpr int kSegs = 10;      // segments alive: one per slot, one being planned, one spare
 
 struct alignas(8) RowsRecord {  // one sensor of a group: window address and row limit (as bits)

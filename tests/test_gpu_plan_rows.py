@@ -230,3 +230,22 @@ def test_shapes_of_computed_delays(tile, dtype):
         _set_weights(bp, 256)
         assert _check_plan([bp], [48], dtype)["fb_mask"] == (16 if dtype == "f32" else 8)
         assert _check_plan([bp], [24], dtype)["smem_budget_kb"] == 110
+
+
+def test_one_long_record_leaves_a_class_its_ctas():
+    """The budget of a class follows its instances' units, not its longest window."""
+    with _handle((160, 160), 130, 401) as many, _handle((24, 24), 8, 6001) as long:
+        assert long.info["window"] > 512
+        info = _check_plan([many, long], [8, 8])
+        assert info["n_classes"] == 1 and info["smem_budget_kb"] == 72
+
+
+@pytest.mark.parametrize("mode", ["table", "constant"])
+@pytest.mark.parametrize("frames", [5, 8, 40])
+def test_one_long_record_leaves_the_groups_of_the_others(mode, frames):
+    """Groups of sensors follow the windows of each tile: an instance whose
+    windows fill a third of the ring or more does not cut those of the others."""
+    with _handle((96, 100), 130, 401, 128, mode) as many, _handle((24, 24), 9, 6001, 128, mode) as long:
+        one = _check_plan([many], [frames])
+        both = _check_plan([many, long], [frames, frames])
+        assert both["fb_mask"] == one["fb_mask"] and both["sensors_per_stage"] == one["sensors_per_stage"]
