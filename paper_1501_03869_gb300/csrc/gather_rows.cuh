@@ -18,8 +18,8 @@
 // and FP32 arithmetic are packed or shared by the frames of a lane.
 // Measured, whole calls (preprocessing and reduction included): 64 FP32 frames
 // of 512 sensors x 21 323 pixels 489 -> 346 us; 8 BF16 frames of 640 sensors x
-// 1.04 M voxels 3.17 -> 2.12 ms; 64 BF16 frames of 64 x 6 092 54 -> 33 us; 12
-// FP16 frames with solid-angle weights 166 -> 136 us.
+// 1.04 M voxels 3.16 -> 2.14 ms; 64 BF16 frames of 64 x 6 092 54 -> 33 us; 12
+// FP16 frames with solid-angle weights 166 -> 134 us.
 //
 // Work: one unit is (frame group, tile) with all segments of G sensors when
 // there are many units, else (frame group, tile, segment), whose sums
@@ -306,6 +306,9 @@ __global__ void __launch_bounds__(RowsShape<P, FB, FMT, MODE>::THREADS, RowsShap
       issue_meta(p.inst[q.inst], q.tile, q.seg0, 0);
       meta_last = 0;
     }
+    // lane k: window rows that a group of k + 1 sensors may have
+    const int room = int(ring_bytes / rows_share(FB) & ~127u) - int(RowsGroup(lane + 1, P, FB, MODE).win);
+    const int cap = lane < p.S && room >= 0 ? room / (FB * 4) : -1;
     bool ok = true;
     int64_t ju = 0;
     int sgi = 0;  // next segment record
@@ -358,8 +361,8 @@ __global__ void __launch_bounds__(RowsShape<P, FB, FMT, MODE>::THREADS, RowsShap
           sg.stride = uint64_t(d.n_t_pad) * ROW;
         }
         __syncwarp();
-        // Groups of up to S sensors as their windows come, each at most a third of
-        // the ring: one long window in a class must not cut every group down to the
+        // Groups of up to S sensors as their windows come, each at most a half or
+        // a third of the ring: one long window in a class must not cut every group down to the
         // two sensors that would fit with it.  They end on whole turns of the phases
         // where there are as many.
         uint32_t before = 0;
@@ -367,8 +370,7 @@ __global__ void __launch_bounds__(RowsShape<P, FB, FMT, MODE>::THREADS, RowsShap
           const int at = i0 + lane;
           const uint32_t u0 = __shfl_sync(0xffffffffu, a0, at & 31), u1 = __shfl_sync(0xffffffffu, a1, at & 31);
           const uint32_t upto = at < 32 ? u0 : u1;  // rows up to this sensor
-          const bool in = lane < p.S && at < n &&
-                          RowsGroup(lane + 1, P, FB, MODE).bytes(int(upto - before), FB) <= ring_bytes / kRowsShare;
+          const bool in = at < n && int(upto - before) <= cap;
           int se = max(1, __popc(__ballot_sync(0xffffffffu, in)));
           const int turn = i0 & (SW - 1);
           if (turn) se = min(se, SW - turn);

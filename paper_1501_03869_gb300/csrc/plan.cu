@@ -4,10 +4,11 @@
 // work to a persistent gather launch.  Instances are grouped by the frames
 // that share one pass over a table tile (FB: the largest power of two up to
 // 8 not above the instance's frame count; 16 or 32 above 16 frames where that
-// pads no further and choose_frames_per_unit finds it faster), and every group ("class") has its own preprocessing launch
-// (the Eq. (BP) integrand of all its instances), its own gather launch and,
-// from 4 frames per unit on, the launch that adds its segments; all
-// preprocessing launches go first, then the gathers.  A 16-frame instance
+// pads no further, the class fills the chip and windows are short enough), and
+// every group ("class") has its own preprocessing launch (the Eq. (BP)
+// integrand of all its instances), its own gather launch and, from 4 frames per
+// unit on, the launch that adds its segments; all preprocessing launches go
+// first, then the gathers.  A 16-frame instance
 // therefore streams its table twice, while a single-frame instance next to it
 // does not pay for frames it does not have.
 // A plan can replay the launches as a CUDA graph whose kernel-node parameters

@@ -2,7 +2,7 @@
 // plain C++ so that a host test can check it (internal).
 //
 // Header, then a ring of StreamParams::ring bytes that is filled with groups of
-// S consecutive sensors (kSlots of them at most), then 2 zero rows that
+// up to S consecutive sensors (kSlots groups at most), then 2 zero rows that
 // out-of-record pixels read, then the running sums of whole-tile units.  A
 // group takes the bytes it needs: windows differ threefold between tiles and
 // sensors, and fixed stages sized for the longest sum left two or three stages
@@ -30,7 +30,12 @@ namespace patbp {
 
 constexpr int kSlots = 8;
 constexpr int kRowsMaxS = 16;  // sensors of a group
-constexpr int kRowsShare = 3;  // a group of several sensors takes at most this part of the ring
+// A group of several sensors takes at most this part of the ring.  Fewer, larger
+// groups win where rows are short (12 BF16 frames in rows of 8, 120 tiles: half the
+// ring 33.3 us, a third 35.3; only 32 uneven instances would have it otherwise, 2.58
+// and 2.54 ms), more groups in flight where they are long (12 and 32 frames of that
+// series in rows of 16 and 32: half 0.7 and 1.2 % slower; a quarter loses in both).
+PATBP_HD constexpr int rows_share(int FB) { return FB >= 16 ? 3 : 2; }
 constexpr int kSegs = 10;      // segments alive: one per slot, one being planned, one spare
 
 struct alignas(8) RowsRecord {  // one sensor of a group: window address and row limit (as bits)
