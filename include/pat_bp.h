@@ -294,7 +294,8 @@ pat_status pat_table_host(const float* speed_host, const pat_grid* grid, const d
  * counts and frame counts).  A plan fixes the handles and their frame counts
  * and groups the instances by frames per unit FB (the largest power of two up
  * to 8 not above an instance's frame count; 16 or 32 above 16 frames where that
- * pads no further: FB frames share each pass over a table tile).  Each
+ * pads no further, its windows are short enough and the group fills the device:
+ * FB frames share each pass over a table tile).  Each
  * execution runs one preprocessing launch per group, then one persistent gather
  * launch per group (the first programmatically dependent on the preprocessing;
  * from 4 frames on followed by the segment sums), optionally replayed as a CUDA graph.  The

@@ -17,9 +17,9 @@
 // this one 1.57 and 1.62, counted from the tables' rows).  Index arithmetic
 // and FP32 arithmetic are packed or shared by the frames of a lane.
 // Measured, whole calls (preprocessing and reduction included): 64 FP32 frames
-// of 512 sensors x 21 323 pixels 489 -> 346 us; 8 BF16 frames of 640 sensors x
+// of 512 sensors x 21 323 pixels 489 -> 317 us; 8 BF16 frames of 640 sensors x
 // 1.04 M voxels 3.16 -> 2.14 ms; 64 BF16 frames of 64 x 6 092 54 -> 33 us; 12
-// FP16 frames with solid-angle weights 166 -> 134 us.
+// FP16 frames with solid-angle weights 166 -> 127 us.
 //
 // Work: one unit is (frame group, tile) with all segments of G sensors when
 // there are many units, else (frame group, tile, segment), whose sums
